@@ -76,8 +76,11 @@ void launch_filter_inst(cudaStream_t st, const int* la_c, const int* la_i, const
                         const unsigned int* mark, Counters* cnt_c, int* lc_c, int* lc_i, int nblocks);
 void launch_count_fail(cudaStream_t st, const unsigned int* fail, int n_inst, unsigned long long* total);
 cudaError_t upload_tables_parent(const dgt::Tabs* tabs);
-void launch_parent(int dim, int pde, int N, const LaunchArgs& a, const int* lc, const int* li, const Counters* cnt,
-                   double* lim, int nblocks);
+cudaError_t upload_tables_lim2(const dgt::Tabs* tabs, const dgt::Tabs* ptabs);
+void launch_parent1(int pde, int N, const LaunchArgs& a, const int* lc, const int* li, const Counters* cnt, double* lim,
+                    int nblocks);
+void launch_parent2(int pde, int N, const LaunchArgs& a, const int* lc, const int* li, const Counters* cnt, double* lim,
+                    int nblocks);
 void launch_kxrcf(int dim, int pde, int N, const LaunchArgs& a, const double* hpow, const double* psi_m1,
                   const double* psi_p1, const double* psi_q, const double* gw, unsigned char* flags, Counters* cnt,
                   int* lc, int* li);
@@ -136,6 +139,7 @@ dg_status dg_ensure_tables_internal() {
   CK(upload_tables1(g_tabs));
   CK(upload_tables2(g_tabs));
   CK(upload_tables_parent(g_ptabs));
+  CK(upload_tables_lim2(g_tabs, g_ptabs));
   done.push_back(dev);
   g_tables_dev = dev;
   return DG_OK;
@@ -659,7 +663,8 @@ static void k_flag(dg_mesh* m, double M) {
 
 static void k_parent_list(dg_mesh* m, const int* lc, const int* li, const Counters* cnt) {
   auto a = args<LaunchArgs>(m, 0, m->cur, m->cur);
-  launch_parent(m->dim, m->pde, m->N, a, lc, li, cnt, m->lim, m->limit_blocks);
+  if (m->dim == 1) launch_parent1(m->pde, m->N, a, lc, li, cnt, m->lim, m->limit_blocks);
+  else launch_parent2(m->pde, m->N, a, lc, li, cnt, m->lim, m->limit_blocks);
   if (m->dim == 1) launch_scatter1(m->pde, m->N, a, m->lim, lc, cnt, m->limit_blocks);
   else launch_scatter2(m->pde, m->N, a, m->lim, lc, cnt, m->limit_blocks);
   m->launches += 2;

@@ -7,8 +7,6 @@
 //   k_stage2    the same stage fused in one kernel per tile (halo warps, shared faces),
 //               an autotuner alternative
 //   k_flag2     TVB minmod indicator + ballot/scan compaction of troubled cells
-//   k_limit2    CSWENO limiter (Sec. 3): Burgers one thread per troubled cell, Euler
-//               four lanes per troubled cell (k_limit2_euler_quad)
 //   k_project2  initial L2 projection (Eq. (2))
 //   k_speed2    largest characteristic speed over the cell means
 //
@@ -28,18 +26,14 @@ constexpr int TY = 8;   // rows per tile of the indicator and projection kernels
 // ----------------------------------------------------------------------------- tables
 template <int N>
 struct Lay {
-  static constexpr int Q = N + 1, NP = (N + 1) * (N + 2) / 2, NS = 2 * N + 1, NG = (N == 1 ? 2 : 4);
+  static constexpr int Q = N + 1, NP = (N + 1) * (N + 2) / 2;
   static constexpr int N1 = N + 1;
   static constexpr int SIZE_DG = 3 * Q * Q * NP + N1 + 2 * Q * N1;
   static constexpr int SIZE_FLAG = 4 * NP + 1;
-  static constexpr int SIZE_LIM = NS * N1 + N1 * NG * N1 + NG * N1 + N1 * N1 * N1 + NG * N1 + NG +
-                                  2 * NG * N1 + 3 * NG;
   static constexpr int SIZE_PROJ = 3 * 8 + 8 * N1;
   static constexpr int SIZE_SPLIT = Q * N1;
-  static constexpr int SIZE_LIM2 = N1 * (N * N1 / 2) + NG * N1;
   static constexpr int SIZE_K = Q * N1 + N1;
-  static constexpr int SIZE_LIM3 = N1 * NG * N1;
-  static constexpr int SIZE = SIZE_DG + SIZE_FLAG + SIZE_LIM + SIZE_PROJ + SIZE_SPLIT + SIZE_LIM2 + SIZE_K + SIZE_LIM3;
+  static constexpr int SIZE = SIZE_DG + SIZE_FLAG + SIZE_PROJ + SIZE_SPLIT + SIZE_K;
 };
 __host__ __device__ constexpr int base_of(int N) {
   return N == 1 ? 0 : (N == 2 ? Lay<1>::SIZE : Lay<1>::SIZE + Lay<2>::SIZE);
@@ -47,7 +41,7 @@ __host__ __device__ constexpr int base_of(int N) {
 template <int N>
 struct Off {
   using L = Lay<N>;
-  static constexpr int Q = L::Q, NP = L::NP, NS = L::NS, NG = L::NG, N1 = L::N1;
+  static constexpr int Q = L::Q, NP = L::NP, N1 = L::N1;
   static constexpr int VP = base_of(N);          // [Q*Q][NP] psi_a(x_qx) psi_b(x_qy)
   static constexpr int VDX = VP + Q * Q * NP;    // w w psi_a'(x_qx) psi_b(x_qy)
   static constexpr int VDY = VDX + Q * Q * NP;   // w w psi_a(x_qx) psi_b'(x_qy)
@@ -59,28 +53,14 @@ struct Off {
   static constexpr int TN = TW + NP;             // psi_a(0) psi_b(1)
   static constexpr int TS = TN + NP;             // psi_a(0) psi_b(-1)
   static constexpr int C00 = TS + NP;            // psi_0(0)^2
-  static constexpr int SA = C00 + 1;             // [NS][N1]
-  static constexpr int WC = SA + NS * N1;        // [N1 stencil][NG][N1]
-  static constexpr int GAM = WC + N1 * NG * N1;  // [NG][N1]
-  static constexpr int BB = GAM + NG * N1;       // [N1][N1][N1]
-  static constexpr int PG = BB + N1 * N1 * N1;   // [NG][N1] psi_n(r_g)
-  static constexpr int WG = PG + NG * N1;        // [NG]
-  static constexpr int GPN = WG + NG;            // [NG][N1]
-  static constexpr int GMN = GPN + NG * N1;      // [NG][N1]
-  static constexpr int SGP = GMN + NG * N1;      // [NG]
-  static constexpr int SGM = SGP + NG;           // [NG]
-  static constexpr int NEG = SGM + NG;           // [NG] 1.0 where a weight is negative
-  static constexpr int PX = NEG + NG;            // [8]
+  static constexpr int PX = C00 + 1;             // [8]
   static constexpr int PW = PX + 8;              // [8]
   static constexpr int PQP = PW + 8;             // [8] (count in slot 0)
   static constexpr int PP = PQP + 8;             // [8][N1]
   static constexpr int WDQ = PP + 8 * N1;        // [Q][N1] w_q psi_n'(x_q)
-  static constexpr int BD = WDQ + Q * N1;        // [N1][j <= j'] Eq. (13) on differences (see pack)
-  static constexpr int WPG = BD + N1 * (N * N1 / 2);  // [NG][N1] w_g psi_n(r_g)
-  static constexpr int KQ = WPG + NG * N1;       // [Q][N1] sqrt(2) psi_n(x_q) = psi_n(x_q) / psi_0
+  static constexpr int KQ = WDQ + Q * N1;        // [Q][N1] sqrt(2) psi_n(x_q) = psi_n(x_q) / psi_0
   static constexpr int KP1 = KQ + Q * N1;        // [N1] sqrt(2) psi_n(1)
-  static constexpr int WCG = KP1 + N1;           // [N1 stencil][NG][N1] gamma_gi C_igk
-  static constexpr int END = WCG + N1 * NG * N1;
+  static constexpr int END = KP1 + N1;
 };
 static_assert(Off<3>::END == Lay<1>::SIZE + Lay<2>::SIZE + Lay<3>::SIZE, "table layout");
 constexpr int kTabSize = Off<3>::END;
@@ -92,7 +72,7 @@ __constant__ double c_tab[kTabSize];
 template <int N>
 void pack(const dgt::Tabs& t, double* h) {
   using O = Off<N>;
-  constexpr int Q = O::Q, NP = O::NP, NS = O::NS, NG = O::NG, N1 = O::N1;
+  constexpr int Q = O::Q, NP = O::NP, N1 = O::N1;
   for (int qy = 0; qy < Q; ++qy)
     for (int qx = 0; qx < Q; ++qx)
       for (int m = 0; m < NP; ++m) {
@@ -116,27 +96,6 @@ void pack(const dgt::Tabs& t, double* h) {
     h[O::TS + m] = t.psi_0[a] * t.psi_m1[b];
   }
   h[O::C00] = t.psi_0[0] * t.psi_0[0];
-  for (int k = 0; k < NS; ++k)
-    for (int n = 0; n < N1; ++n) h[O::SA + k * N1 + n] = t.SA[k][n];
-  for (int i = 0; i < N1; ++i)
-    for (int g = 0; g < NG; ++g)
-      for (int k = 0; k < N1; ++k) h[O::WC + (i * NG + g) * N1 + k] = t.C[i][g][k];
-  for (int g = 0; g < NG; ++g)
-    for (int i = 0; i < N1; ++i) {
-      h[O::GAM + g * N1 + i] = t.gam[g][i];
-      h[O::GPN + g * N1 + i] = t.gpn[g][i];
-      h[O::GMN + g * N1 + i] = t.gmn[g][i];
-    }
-  for (int i = 0; i < N1; ++i)
-    for (int k = 0; k < N1; ++k)
-      for (int l = 0; l < N1; ++l) h[O::BB + (i * N1 + k) * N1 + l] = t.B[i][k][l];
-  for (int g = 0; g < NG; ++g) {
-    for (int n = 0; n < N1; ++n) h[O::PG + g * N1 + n] = t.psiG[g][n];
-    h[O::WG + g] = t.rw[g];
-    h[O::SGP + g] = t.sgp[g];
-    h[O::SGM + g] = t.sgm[g];
-    h[O::NEG + g] = t.neg[g] ? 1.0 : 0.0;
-  }
   for (int q = 0; q < t.QP; ++q) {
     h[O::PX + q] = t.px[q];
     h[O::PW + q] = t.pw[q];
@@ -145,30 +104,9 @@ void pack(const dgt::Tabs& t, double* h) {
   h[O::PQP] = t.QP;
   for (int q = 0; q < Q; ++q)
     for (int n = 0; n < N1; ++n) h[O::WDQ + q * N1 + n] = t.gw[q] * t.dpsi_q[q][n];
-  for (int g = 0; g < NG; ++g)
-    for (int n = 0; n < N1; ++n) h[O::WPG + g * N1 + n] = t.rw[g] * t.psiG[g][n];
   for (int q = 0; q < Q; ++q)
     for (int n = 0; n < N1; ++n) h[O::KQ + q * N1 + n] = t.kq[q][n];
   for (int n = 0; n < N1; ++n) h[O::KP1 + n] = t.kp1[n];
-  // beta_i as a quadratic form in the N differences d_j = x_{i+j+1} - x_{i+j} of the
-  // stencil's averages x (beta ignores constants): with x_{i+k} - x_i = sum_{j<k} d_j,
-  // M_jj' = sum_{k > j, l > j'} B_ikl; packed as M_jj and M_jj' + M_j'j (j < j')
-  for (int i = 0; i < N1; ++i) {
-    int j = 0;
-    for (int a = 0; a < N; ++a)
-      for (int b = a; b < N; ++b, ++j) {
-        double mab = 0.0, mba = 0.0;
-        for (int k = a + 1; k < N1; ++k)
-          for (int l = b + 1; l < N1; ++l) {
-            mab += t.B[i][k][l];
-            mba += t.B[i][l][k];
-          }
-        h[O::BD + i * (N * N1 / 2) + j] = a == b ? mab : mab + mba;
-      }
-  }
-  for (int i = 0; i < N1; ++i)
-    for (int g = 0; g < NG; ++g)
-      for (int k = 0; k < N1; ++k) h[O::WCG + (i * NG + g) * N1 + k] = t.gam[g][i] * t.C[i][g][k];
 }
 
 // ----------------------------------------------------------------------------- loads
@@ -1123,434 +1061,6 @@ __global__ void __launch_bounds__(256)
   block_compact(fl, near ? 1 : 0, g, tile.inst, cnt, list_cell, list_inst);
 }
 
-// ----------------------------------------------------------------------------- limiter
-// One WENO reconstruction (Sec. 3, Steps 2-5) from the 2N+1 stencil averages to the NG
-// Step 1 points.  Eq. (14) read as wbar_i = gamma_i / (eps + beta_i)^2; where a linear
-// weight is negative (P3) the split gamma = sigma+ gamma~+ - sigma- gamma~- of Shi, Hu and
-// Shu is used, each part normalised separately.
-template <int N>
-__device__ __forceinline__ void weno(const double* avg, double* out) {
-  using O = Off<N>;
-  constexpr int N1 = N + 1, NG = O::NG;
-  const double eps = 1e-6;
-  // p_i - c does not change when a constant c is removed from all averages (constants are
-  // reproduced): work on averages centred at the troubled cell's own
-  const double c = avg[N];
-  double dv[2 * N + 1];
-#pragma unroll
-  for (int k = 0; k < 2 * N + 1; ++k) dv[k] = avg[k] - c;
-  // Eq. (13) holds only derivatives, so beta_i is a quadratic form in the differences of
-  // the stencil's averages: beta_i = sum_j df_{i+j} sum_{j' >= j} Md_jj' df_{i+j'};
-  // inv_i = 1 / (eps + beta_i)^2
-  constexpr int ND = N * N1 / 2;
-  double df[2 * N];
-#pragma unroll
-  for (int k = 0; k < 2 * N; ++k) df[k] = avg[k + 1] - avg[k];
-  double inv[N1];
-#pragma unroll
-  for (int i = 0; i < N1; ++i) {
-    double beta = 0.0;
-    int j = 0;
-#pragma unroll
-    for (int k = 0; k < N; ++k) {
-      double r = T(O::BD + i * ND + j) * df[i + k];
-      ++j;
-#pragma unroll
-      for (int l = k + 1; l < N; ++l, ++j) r = fma(T(O::BD + i * ND + j), df[i + l], r);
-      beta = k == 0 ? df[i] * r : fma(df[i + k], r, beta);
-    }
-    const double d = eps + beta;
-    inv[i] = rcp_d(d * d);
-  }
-  // Eqs. (14)-(15): u_g = c + sum_i wbar_i (p_i - c) / sum_i wbar_i, wbar_i = gamma_gi inv_i;
-  // with the linear weights folded into the reconstruction tables (WCG = gamma_gi C_igk)
-  // the numerator is sum_i inv_i (gamma_gi (p_i - c))
-#pragma unroll
-  for (int g = 0; g < NG; ++g) {
-    if (T(O::NEG + g) == 0.0) {
-      double sw = 0.0, su = 0.0;
-#pragma unroll
-      for (int i = 0; i < N1; ++i) {
-        double s = T(O::WCG + (i * NG + g) * N1) * dv[i];
-#pragma unroll
-        for (int k = 1; k < N1; ++k) s = fma(T(O::WCG + (i * NG + g) * N1 + k), dv[i + k], s);
-        sw = i == 0 ? T(O::GAM + g * N1) * inv[0] : fma(T(O::GAM + g * N1 + i), inv[i], sw);
-        su = i == 0 ? inv[0] * s : fma(inv[i], s, su);
-      }
-      out[g] = fma(su, rcp_d(sw), c);
-    } else {
-      double p[N1];
-#pragma unroll
-      for (int i = 0; i < N1; ++i) {
-        double s = T(O::WC + (i * NG + g) * N1) * dv[i];
-#pragma unroll
-        for (int k = 1; k < N1; ++k) s = fma(T(O::WC + (i * NG + g) * N1 + k), dv[i + k], s);
-        p[i] = s;
-      }
-      double swp = 0.0, sup = 0.0, swm = 0.0, sum = 0.0;
-#pragma unroll
-      for (int i = 0; i < N1; ++i) {
-        const double wp = T(O::GPN + g * N1 + i) * inv[i];
-        const double wm = T(O::GMN + g * N1 + i) * inv[i];
-        swp += wp;
-        sup = fma(wp, p[i], sup);
-        swm += wm;
-        sum = fma(wm, p[i], sum);
-      }
-      // sigma+ - sigma- = 1: the constant c passes through the split unchanged
-      out[g] = c + (T(O::SGP + g) * (sup * rcp_d(swp)) - T(O::SGM + g) * (sum * rcp_d(swm)));
-    }
-  }
-}
-
-// Right/left eigenvectors of the 2D Euler flux Jacobian in direction dir at state u.
-__device__ __forceinline__ void euler_eig2(const double* u, int dir, double gam, double (&R)[4][4],
-                                           double (&L)[4][4]) {
-  const double rho = u[0], r = rcp_d(rho);
-  const double vx = u[1] * r, vy = u[2] * r, q2 = vx * vx + vy * vy;
-  const double p = (gam - 1.0) * (u[3] - 0.5 * rho * q2);
-  const double c = sqrt_d(gam * p * r), ic = rcp_d(c);
-  const double H = (u[3] + p) * r;
-  const double b1 = (gam - 1.0) * ic * ic, b2 = 0.5 * b1 * q2;
-  const double vn = dir == 0 ? vx : vy, vt = dir == 0 ? vy : vx;
-  const int in = dir == 0 ? 1 : 2, it = dir == 0 ? 2 : 1;
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) { R[i][j] = 0.0; L[i][j] = 0.0; }
-  R[0][0] = 1.0; R[in][0] = vn - c; R[it][0] = vt; R[3][0] = H - vn * c;
-  R[0][1] = 1.0; R[in][1] = vn;     R[it][1] = vt; R[3][1] = 0.5 * q2;
-  R[it][2] = 1.0; R[3][2] = vt;
-  R[0][3] = 1.0; R[in][3] = vn + c; R[it][3] = vt; R[3][3] = H + vn * c;
-  L[0][0] = 0.5 * (b2 + vn * ic); L[0][in] = -0.5 * (b1 * vn + ic); L[0][it] = -0.5 * b1 * vt; L[0][3] = 0.5 * b1;
-  L[1][0] = 1.0 - b2;             L[1][in] = b1 * vn;               L[1][it] = b1 * vt;        L[1][3] = -b1;
-  L[2][0] = -vt;                  L[2][it] = 1.0;
-  L[3][0] = 0.5 * (b2 - vn * ic); L[3][in] = 0.5 * (ic - b1 * vn);  L[3][it] = -0.5 * b1 * vt; L[3][3] = 0.5 * b1;
-}
-
-// CSWENO on the listed cells; thread i handles list entry i.  Output: the limited modes
-// 1..NP-1 in list order (lim[(v*NP + m) * cap + i]).
-template <int PDE, int N>
-__global__ void __launch_bounds__(128)
-    k_limit2(const double* __restrict__ U, const Inst* __restrict__ insts, long long ctot, int bc,
-             const int* __restrict__ list_cell, const int* __restrict__ list_inst, const Counters* __restrict__ cnt,
-             double* __restrict__ lim, long long cap, double gam) {
-  using O = Off<N>;
-  constexpr int V = nv_of(2, PDE), NP = np_of(2, N), NS = O::NS, NG = O::NG, N1 = N + 1;
-  const unsigned int n = cnt->n_flag;
-  for (unsigned int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const long long g = list_cell[i];
-    const Inst I = insts[list_inst[i]];
-    const int loc = (int)(g - I.off);
-    const int ix = loc % I.nx, iy = loc / I.nx;
-    // (2N+1)^2 sub-rectangle averages of the 3x3 neighbourhood (Fig. 1 in each direction)
-    double avg[V][NS][NS];
-#pragma unroll
-    for (int dy = -1; dy <= 1; ++dy)
-#pragma unroll
-      for (int dx = -1; dx <= 1; ++dx) {
-        double u[V][NP];
-        load_cell<V, NP>(U, ctot, I, ix + dx, iy + dy, bc, u);
-        constexpr int k0[3] = {0, N, N + 1};
-        constexpr int kn[3] = {N, 1, N};
-#pragma unroll
-        for (int v = 0; v < V; ++v)
-#pragma unroll
-          for (int kx = k0[dx + 1]; kx < k0[dx + 1] + kn[dx + 1]; ++kx) {
-            double t[N1];  // t_b = sum_a U_ab SA[kx][a]
-#pragma unroll
-            for (int b = 0; b <= N; ++b) {
-              double s = 0.0;
-#pragma unroll
-              for (int a = 0; a <= N - b; ++a) s = fma(u[v][mode_idx(a, b)], T(O::SA + kx * N1 + a), s);
-              t[b] = s;
-            }
-#pragma unroll
-            for (int ky = k0[dy + 1]; ky < k0[dy + 1] + kn[dy + 1]; ++ky) {
-              double s = 0.0;
-#pragma unroll
-              for (int b = 0; b <= N; ++b) s = fma(t[b], T(O::SA + ky * N1 + b), s);
-              avg[v][ky][kx] = s;
-            }
-          }
-      }
-    // x sweep: rowval[v][ky][g] = average over row ky of u(x_g, y)
-    double rowv[V][NS][NG];
-    double pv[V][NG][NG];  // [v][gy][gx]
-    if constexpr (PDE == 1) {
-      double mean[4];
-#pragma unroll
-      for (int v = 0; v < 4; ++v) mean[v] = __ldg(U + (long long)(v * NP) * ctot + g) * T(O::C00);
-      double R[4][4], L[4][4];
-      euler_eig2(mean, 0, gam, R, L);
-#pragma unroll
-      for (int ky = 0; ky < NS; ++ky) {
-        double wv[4][NG];
-#pragma unroll
-        for (int f = 0; f < 4; ++f) {
-          double wc[NS];
-#pragma unroll
-          for (int kx = 0; kx < NS; ++kx) {
-            double s = 0.0;
-#pragma unroll
-            for (int v = 0; v < 4; ++v)
-              s = fma(L[f][v], avg[v][ky][kx], s);
-            wc[kx] = s;
-          }
-          weno<N>(wc, wv[f]);
-        }
-#pragma unroll
-        for (int v = 0; v < 4; ++v)
-#pragma unroll
-          for (int q = 0; q < NG; ++q) {
-            double s = 0.0;
-#pragma unroll
-            for (int f = 0; f < 4; ++f) s = fma(R[v][f], wv[f][q], s);
-            rowv[v][ky][q] = s;
-          }
-      }
-      euler_eig2(mean, 1, gam, R, L);
-#pragma unroll
-      for (int gx = 0; gx < NG; ++gx) {
-        double wv[4][NG];
-#pragma unroll
-        for (int f = 0; f < 4; ++f) {
-          double wc[NS];
-#pragma unroll
-          for (int ky = 0; ky < NS; ++ky) {
-            double s = 0.0;
-#pragma unroll
-            for (int v = 0; v < 4; ++v) s = fma(L[f][v], rowv[v][ky][gx], s);
-            wc[ky] = s;
-          }
-          weno<N>(wc, wv[f]);
-        }
-#pragma unroll
-        for (int v = 0; v < 4; ++v)
-#pragma unroll
-          for (int gy = 0; gy < NG; ++gy) {
-            double s = 0.0;
-#pragma unroll
-            for (int f = 0; f < 4; ++f) s = fma(R[v][f], wv[f][gy], s);
-            pv[v][gy][gx] = s;
-          }
-      }
-    } else {
-#pragma unroll
-      for (int ky = 0; ky < NS; ++ky) weno<N>(avg[0][ky], rowv[0][ky]);
-#pragma unroll
-      for (int gx = 0; gx < NG; ++gx) {
-        double col[NS], r[NG];
-#pragma unroll
-        for (int ky = 0; ky < NS; ++ky) col[ky] = rowv[0][ky][gx];
-        weno<N>(col, r);
-#pragma unroll
-        for (int gy = 0; gy < NG; ++gy) pv[0][gy][gx] = r[gy];
-      }
-    }
-    // Step 6 (Eq. (16)) with the tensor rule: U_ab = sum w_gx w_gy u psi_a(x_gx) psi_b(y_gy)
-#pragma unroll
-    for (int v = 0; v < V; ++v) {
-      double tq[NG][N1];  // tq[gy][a] = sum_gx w_gx psi_a(x_gx) pv[gy][gx]
-#pragma unroll
-      for (int gy = 0; gy < NG; ++gy)
-#pragma unroll
-        for (int a = 0; a <= N; ++a) {
-          double s = 0.0;
-#pragma unroll
-          for (int gx = 0; gx < NG; ++gx) s = fma(T(O::WPG + gx * N1 + a), pv[v][gy][gx], s);
-          tq[gy][a] = s;
-        }
-#pragma unroll
-      for (int m = 1; m < NP; ++m) {
-        const int a = mode_a(m), b = mode_b(m);
-        double s = 0.0;
-#pragma unroll
-        for (int gy = 0; gy < NG; ++gy) s = fma(T(O::WPG + gy * N1 + b), tq[gy][a], s);
-        lim[(long long)(v * NP + m) * cap + i] = s;
-      }
-    }
-  }
-}
-
-
-// CSWENO for 2D Euler with four lanes per troubled cell (8 cells per warp).  Lane q of a
-// quad owns conserved variable q for the subcell averages and the projection, and
-// characteristic field q in the two sweeps; the quad exchanges values with shuffles, so
-// all lanes run the same FP64 instruction stream (the FP64 pipe is the bottleneck) while
-// each thread holds a quarter of the per-cell state.  With a work counter (lq, zero at
-// launch) every warp takes its next 8 cells from it, so the work spreads evenly over the
-// resident warps whatever the grid; without one the warps stride over the list.
-template <int N>
-__global__ void __launch_bounds__(128)
-    k_limit2_euler_quad(const double* __restrict__ U, const Inst* __restrict__ insts, long long ctot, int bc,
-                        const int* __restrict__ list_cell, const int* __restrict__ list_inst,
-                        const Counters* __restrict__ cnt, double* __restrict__ lim, long long cap, double gam,
-                        unsigned int* __restrict__ lq, const double* __restrict__ bcd) {
-  using O = Off<N>;
-  constexpr int NP = np_of(2, N), NS = O::NS, NG = O::NG, N1 = N + 1;
-  const unsigned int n = cnt->n_flag;
-  const int lane = threadIdx.x & 31, q = lane & 3, qb = lane & ~3;
-  const unsigned int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const unsigned int nwarps = (gridDim.x * blockDim.x) >> 5;
-  for (unsigned int it = 0;; ++it) {
-    unsigned int base;
-    if (lq) {
-      unsigned int b0 = 0;
-      if (lane == 0) b0 = atomicAdd(lq, 8u);
-      base = __shfl_sync(0xffffffffu, b0, 0);
-    } else {
-      base = (warp + it * nwarps) * 8u;
-    }
-    if (base >= n) break;
-    const unsigned int i0 = base + (lane >> 2);
-    const bool active = i0 < n;
-    const unsigned int i = active ? i0 : n - 1;  // idle quads repeat a valid entry
-    const long long g = list_cell[i];
-    const int inst = list_inst[i];
-    const Inst I = insts[inst];
-    const int loc = (int)(g - I.off);
-    const int ix = loc % I.nx, iy = loc / I.nx;
-    // subcell averages of variable q
-    double avg[NS][NS];
-#pragma unroll
-    for (int dy = -1; dy <= 1; ++dy)
-#pragma unroll
-      for (int dx = -1; dx <= 1; ++dx) {
-        int jx = ix + dx, jy = iy + dy;
-        bool fx = false, fy = false, fv = false;
-        const double* cst = nullptr;  // kBcDmr constant ghost
-        if (bc == 0) {
-          jx = jx < 0 ? jx + I.nx : (jx >= I.nx ? jx - I.nx : jx);
-          jy = jy < 0 ? jy + I.ny : (jy >= I.ny ? jy - I.ny : jy);
-        } else if (bc == kBcDmr && (jx < 0 || jx >= I.nx || jy < 0 || jy >= I.ny)) {
-          const Ghost gh = dmr_ghost(I, inst, jx, jy, bcd, dmr_time(bcd, inst, 0));
-          cst = gh.c;
-          jx = gh.jx;
-          jy = gh.jy;
-          fx = gh.fx;
-          fy = gh.fy;
-          fv = gh.fv && q == 2;
-          if (cst) { jx = 0; jy = 0; }
-        } else {
-          if (jx < 0) { jx = 0; fx = true; }
-          if (jx >= I.nx) { jx = I.nx - 1; fx = true; }
-          if (jy < 0) { jy = 0; fy = true; }
-          if (jy >= I.ny) { jy = I.ny - 1; fy = true; }
-        }
-        const long long gj = I.off + (long long)jy * I.nx + jx;
-        double u[NP];
-#pragma unroll
-        for (int m = 0; m < NP; ++m) {
-          const double x = __ldg(U + (long long)(q * NP + m) * ctot + gj);
-          const bool flip = ((fx && (mode_a(m) & 1)) != (fy && (mode_b(m) & 1))) != fv;
-          u[m] = neg_if(x, flip);
-          if (cst) u[m] = m == 0 ? 2.0 * cst[q] : 0.0;
-        }
-        constexpr int k0[3] = {0, N, N + 1};
-        constexpr int kn[3] = {N, 1, N};
-#pragma unroll
-        for (int kx = k0[dx + 1]; kx < k0[dx + 1] + kn[dx + 1]; ++kx) {
-          double t[N1];
-#pragma unroll
-          for (int b = 0; b <= N; ++b) {
-            double sum = 0.0;
-#pragma unroll
-            for (int a = 0; a <= N - b; ++a) sum = fma(u[mode_idx(a, b)], T(O::SA + kx * N1 + a), sum);
-            t[b] = sum;
-          }
-#pragma unroll
-          for (int ky = k0[dy + 1]; ky < k0[dy + 1] + kn[dy + 1]; ++ky) {
-            double sum = 0.0;
-#pragma unroll
-            for (int b = 0; b <= N; ++b) sum = fma(t[b], T(O::SA + ky * N1 + b), sum);
-            avg[ky][kx] = sum;
-          }
-        }
-      }
-    // mean state of the troubled cell, gathered over the quad
-    const double mq = __ldg(U + (long long)(q * NP) * ctot + g) * T(O::C00);
-    double mean[4];
-#pragma unroll
-    for (int v = 0; v < 4; ++v) mean[v] = __shfl_sync(0xffffffffu, mq, qb | v);
-    double Lq[4], Rq[4];  // row q of the left and right eigenvector matrices
-    auto rows_of = [&](int dir) {
-      double R[4][4], L[4][4];
-      euler_eig2(mean, dir, gam, R, L);
-#pragma unroll
-      for (int v = 0; v < 4; ++v) {
-        Lq[v] = q == 0 ? L[0][v] : (q == 1 ? L[1][v] : (q == 2 ? L[2][v] : L[3][v]));
-        Rq[v] = q == 0 ? R[0][v] : (q == 1 ? R[1][v] : (q == 2 ? R[2][v] : R[3][v]));
-      }
-    };
-    // x sweep: field q of each row, back to variable q at the NG x points
-    rows_of(0);
-    double rowv[NS][NG];
-#pragma unroll
-    for (int ky = 0; ky < NS; ++ky) {
-      double w[NS], r[NG];
-#pragma unroll
-      for (int kx = 0; kx < NS; ++kx) {
-        double s = 0.0;
-#pragma unroll
-        for (int v = 0; v < 4; ++v) s = fma(Lq[v], __shfl_sync(0xffffffffu, avg[ky][kx], qb | v), s);
-        w[kx] = s;
-      }
-      weno<N>(w, r);
-#pragma unroll
-      for (int gx = 0; gx < NG; ++gx) {
-        double s = 0.0;
-#pragma unroll
-        for (int f = 0; f < 4; ++f) s = fma(Rq[f], __shfl_sync(0xffffffffu, r[gx], qb | f), s);
-        rowv[ky][gx] = s;
-      }
-    }
-    // y sweep: field q of each x point's column, back to variable q at the NG y points
-    rows_of(1);
-    double pv[NG][NG];  // [gy][gx]
-#pragma unroll
-    for (int gx = 0; gx < NG; ++gx) {
-      double w[NS], r[NG];
-#pragma unroll
-      for (int ky = 0; ky < NS; ++ky) {
-        double s = 0.0;
-#pragma unroll
-        for (int v = 0; v < 4; ++v) s = fma(Lq[v], __shfl_sync(0xffffffffu, rowv[ky][gx], qb | v), s);
-        w[ky] = s;
-      }
-      weno<N>(w, r);
-#pragma unroll
-      for (int gy = 0; gy < NG; ++gy) {
-        double s = 0.0;
-#pragma unroll
-        for (int f = 0; f < 4; ++f) s = fma(Rq[f], __shfl_sync(0xffffffffu, r[gy], qb | f), s);
-        pv[gy][gx] = s;
-      }
-    }
-    // Step 6 for variable q (tensor Gauss / Gauss-Lobatto rule)
-    double tq[NG][N1];
-#pragma unroll
-    for (int gy = 0; gy < NG; ++gy)
-#pragma unroll
-      for (int a = 0; a <= N; ++a) {
-        double s = 0.0;
-#pragma unroll
-        for (int gx = 0; gx < NG; ++gx) s = fma(T(O::WPG + gx * N1 + a), pv[gy][gx], s);
-        tq[gy][a] = s;
-      }
-    if (active) {
-#pragma unroll
-      for (int m = 1; m < NP; ++m) {
-        const int a = mode_a(m), b = mode_b(m);
-        double s = 0.0;
-#pragma unroll
-        for (int gy = 0; gy < NG; ++gy) s = fma(T(O::WPG + gy * N1 + b), tq[gy][a], s);
-        lim[(long long)(q * NP + m) * cap + i] = s;
-      }
-    }
-  }
-}
-
 // ----------------------------------------------------------------------------- projection
 // Eq. (2) for the initial data: U_ab = sum_{qx,qy} w w u0(x, y) psi_a psi_b with N+4 Gauss
 // points per direction.  Parameters per instance (see dg.h for the families).
@@ -1705,19 +1215,6 @@ void launch_flag2(int pde, int N, const LaunchArgs& a, double M, unsigned char* 
                   int* li) {
   DG_DISPATCH2(pde, N, (k2::k_flag2<P_, N_><<<a.ntiles, 256, 0, a.st>>>(a.us, a.inst, a.tiles, a.ctot, a.bc, M,
                                                                           flags, cnt, lc, li, a.bcd)));
-}
-
-void launch_limit2(int pde, int N, const LaunchArgs& a, const int* lc, const int* li, const Counters* cnt,
-                   double* lim, int nblocks) {
-  if (pde == 1) {  // Euler: four lanes per troubled cell
-    if (a.lq) cudaMemsetAsync(a.lq, 0, sizeof(unsigned int), a.st);
-    if (N == 1) k2::k_limit2_euler_quad<1><<<nblocks, 128, 0, a.st>>>(a.us, a.inst, a.ctot, a.bc, lc, li, cnt, lim, a.cap, a.gam, a.lq, a.bcd);
-    else if (N == 2) k2::k_limit2_euler_quad<2><<<nblocks, 128, 0, a.st>>>(a.us, a.inst, a.ctot, a.bc, lc, li, cnt, lim, a.cap, a.gam, a.lq, a.bcd);
-    else k2::k_limit2_euler_quad<3><<<nblocks, 128, 0, a.st>>>(a.us, a.inst, a.ctot, a.bc, lc, li, cnt, lim, a.cap, a.gam, a.lq, a.bcd);
-    return;
-  }
-  DG_DISPATCH2(pde, N, (k2::k_limit2<P_, N_><<<nblocks, 128, 0, a.st>>>(a.us, a.inst, a.ctot, a.bc, lc, li, cnt,
-                                                                          lim, a.cap, a.gam)));
 }
 
 void launch_scatter2(int pde, int N, const LaunchArgs& a, const double* lim, const int* lc, const Counters* cnt,

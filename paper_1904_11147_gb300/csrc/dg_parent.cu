@@ -208,77 +208,6 @@ __global__ void __launch_bounds__(128)
   }
 }
 
-template <int PDE, int N>
-__global__ void __launch_bounds__(128)
-    k_parent2(const double* __restrict__ U, const Inst* __restrict__ insts, long long ctot, int bc,
-              const int* __restrict__ list_cell, const int* __restrict__ list_inst, const Counters* __restrict__ cnt,
-              double* __restrict__ lim, long long cap, double gam) {
-  constexpr int V = nv_of(2, PDE), NP = np_of(2, N), NS = 2 * N + 1, NG = N == 1 ? 2 : 4;
-  const PTab& t = c_pt[N - 1];
-  const unsigned int n = cnt->n_flag;
-  for (unsigned int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const long long g = list_cell[i];
-    const Inst I = insts[list_inst[i]];
-    const int loc = (int)(g - I.off);
-    const int ix = loc % I.nx, iy = loc / I.nx;
-    double Rx[V][V], Lx[V][V], Ry[V][V], Ly[V][V];
-    if constexpr (PDE == 1) {
-      double mean[V];
-#pragma unroll
-      for (int v = 0; v < V; ++v) mean[v] = U[(long long)(v * NP) * ctot + g] * t.psi0 * t.psi0;
-      eig<V>(mean, 0, gam, Rx, Lx);
-      eig<V>(mean, 1, gam, Ry, Ly);
-    }
-    // x sweep, row by row: rowv[v][ky][gx] = average over row ky of u(x_gx, y)
-    double rowv[V][NS][NG];
-#pragma unroll
-    for (int ky = 0; ky < NS; ++ky) {
-      const long long row = I.off + (long long)reflect(iy + ky - N, I.ny, bc) * I.nx;
-      double a[V][NS];
-#pragma unroll
-      for (int kx = 0; kx < NS; ++kx) {
-        const long long c = row + reflect(ix + kx - N, I.nx, bc);
-#pragma unroll
-        for (int v = 0; v < V; ++v) a[v][kx] = U[(long long)(v * NP) * ctot + c] * t.psi0 * t.psi0;
-      }
-      double o[V][NG];
-      sweep<PDE, V, N>(t, a, Rx, Lx, o);
-#pragma unroll
-      for (int v = 0; v < V; ++v)
-#pragma unroll
-        for (int q = 0; q < NG; ++q) rowv[v][ky][q] = o[v][q];
-    }
-    // y sweep per x point, then the tensor projection onto the modes 1 <= a+b <= N
-    double acc[V][NP];
-#pragma unroll
-    for (int v = 0; v < V; ++v)
-#pragma unroll
-      for (int m = 0; m < NP; ++m) acc[v][m] = 0.0;
-#pragma unroll
-    for (int gx = 0; gx < NG; ++gx) {
-      double a[V][NS];
-#pragma unroll
-      for (int v = 0; v < V; ++v)
-#pragma unroll
-        for (int ky = 0; ky < NS; ++ky) a[v][ky] = rowv[v][ky][gx];
-      double o[V][NG];
-      sweep<PDE, V, N>(t, a, Ry, Ly, o);
-#pragma unroll
-      for (int v = 0; v < V; ++v)
-#pragma unroll
-        for (int gy = 0; gy < NG; ++gy) {
-          const double w = t.wg[gx] * t.wg[gy] * o[v][gy];
-#pragma unroll
-          for (int m = 1; m < NP; ++m) acc[v][m] = fma(w * t.pg[gx][mode_a(m)], t.pg[gy][mode_b(m)], acc[v][m]);
-        }
-    }
-#pragma unroll
-    for (int v = 0; v < V; ++v)
-#pragma unroll
-      for (int m = 1; m < NP; ++m) lim[(long long)(v * NP + m) * cap + i] = acc[v][m];
-  }
-}
-
 }  // namespace pw
 
 cudaError_t upload_tables_parent(const dgt::Tabs* tabs /* [3], built with parent = true */) {
@@ -309,7 +238,7 @@ cudaError_t upload_tables_parent(const dgt::Tabs* tabs /* [3], built with parent
   return cudaMemcpyToSymbol(pw::c_pt, h, sizeof(h));
 }
 
-void launch_parent(int dim, int pde, int N, const LaunchArgs& a, const int* lc, const int* li, const Counters* cnt,
+void launch_parent1(int pde, int N, const LaunchArgs& a, const int* lc, const int* li, const Counters* cnt,
                    double* lim, int nblocks) {
   // one warp per block, four times the usual grid: the troubled-cell count is known only on
   // the device, and small lists then still spread over all SMs
@@ -320,13 +249,8 @@ void launch_parent(int dim, int pde, int N, const LaunchArgs& a, const int* lc, 
     else if (N == 2) DG_PW(K, P, 2); \
     else DG_PW(K, P, 3); \
   } while (0)
-  if (dim == 1) {
-    if (pde == 0) DG_PW_N(k_parent1, 0);
-    else DG_PW_N(k_parent1, 1);
-  } else {
-    if (pde == 0) DG_PW_N(k_parent2, 0);
-    else DG_PW_N(k_parent2, 1);
-  }
+  if (pde == 0) DG_PW_N(k_parent1, 0);
+  else DG_PW_N(k_parent1, 1);
 #undef DG_PW_N
 #undef DG_PW
 }

@@ -196,6 +196,7 @@ int build_tables(int N, Tabs* t, bool parent) {
     e[2 * N + 1] = 1.5L;
     // (the loop above sets e[N+1] = 0.5, the troubled cell's right edge)
   }
+  ld Eg[kMaxG][kMaxN + 1][kMaxN], Gm[kMaxG][kMaxN + 1], Sp = 0, Sm = 0;
   for (int g = 0; g < t->NG; ++g) {
     ld xi = rp[g] / 2;
     ld Cl[kMaxN + 1][kMaxN + 1];
@@ -227,6 +228,21 @@ int build_tables(int N, Tabs* t, bool parent) {
       if (gm[i] < 0) neg = 1;
     }
     t->neg[g] = neg;
+    for (int i = 0; i <= N; ++i) {
+      Gm[g][i] = gm[i];
+      // coefficient of d_m = avg[m+1] - avg[m] in p_i(x_g) - avg[N]
+      for (int j = 0; j < N; ++j) {
+        const int mm = i + j;
+        ld s = 0;
+        for (int k = 0; k <= N; ++k) {
+          if (mm >= N && i + k > mm) s += Cl[i][k];
+          if (mm < N && i + k <= mm) s -= Cl[i][k];
+        }
+        Eg[g][i][j] = s;
+      }
+      // one negative weight, at the stencil the kernels expect
+      if ((gm[i] < 0) != (weno_neg(N, g, parent) == i)) return 2;
+    }
     // split of Shi, Hu & Shu with theta = 3 where a weight is negative
     ld sp = 0, sm = 0, gp[kMaxN + 1], gn[kMaxN + 1];
     for (int i = 0; i <= N; ++i) {
@@ -237,11 +253,15 @@ int build_tables(int N, Tabs* t, bool parent) {
     }
     t->sgp[g] = (double)sp;
     t->sgm[g] = (double)sm;
+    if (neg) { Sp = sp; Sm = sm; }
     for (int i = 0; i <= N; ++i) {
       t->gpn[g][i] = (double)(gp[i] / sp);
       t->gmn[g][i] = (double)(sm > 0 ? gn[i] / sm : 0);
     }
   }
+  t->qsp[0] = (double)(4 * Sp - Sm - 1);
+  t->qsp[1] = (double)(4 * Sm - Sp + 1);
+  ld Mb[kMaxN + 1];
   // Eq. (13): beta_i = sum_{l=1}^N int_{-1/2}^{1/2} (d^l p_i / dxi^l)^2 dxi
   {
     ld qx[kMaxQ], qw[kMaxQ];
@@ -259,6 +279,41 @@ int build_tables(int N, Tabs* t, bool parent) {
         }
       for (int a = 0; a <= N; ++a)
         for (int b = 0; b <= N; ++b) t->B[i][a][b] = (double)Bl[a][b];
+      // the form in the differences: with avg[i+k] - avg[i] = sum_{j<k} d_{i+j},
+      // Q_jj' = sum_{k>j, l>j'} B_kl, then e_0 (the far end) completed to a square first
+      ld Q[kMaxN][kMaxN];
+      for (int a = 0; a < N; ++a)
+        for (int b = 0; b < N; ++b) {
+          const int ja = 2 * i <= N ? a : N - 1 - a, jb = 2 * i <= N ? b : N - 1 - b;
+          Q[a][b] = 0;
+          for (int k = ja + 1; k <= N; ++k)
+            for (int l = jb + 1; l <= N; ++l) Q[a][b] += Bl[k][l];
+        }
+      const ld M = Q[0][0];
+      ld f[6] = {1e-6L / M, 0, 0, 0, 0, 0};
+      if (N == 2) {
+        f[3] = Q[0][1] / M;
+        f[1] = (Q[1][1] - Q[0][1] * f[3]) / M;
+      } else if (N == 3) {
+        f[3] = Q[0][1] / M;
+        f[4] = Q[0][2] / M;
+        const ld q11 = Q[1][1] - Q[0][1] * f[3], q12 = Q[1][2] - Q[0][1] * f[4];
+        f[2] = q11 / M;
+        f[5] = q12 / q11;
+        f[1] = (Q[2][2] - Q[0][2] * f[4] - q12 * f[5]) / M;
+      }
+      Mb[i] = M;
+      if (2 * i <= N)
+        for (int c = 0; c < 6; ++c) t->bform[i][c] = (double)f[c];
+    }
+  }
+  for (int g = 0; g < t->NG; ++g) {
+    const int r = weno_ref(N, g);
+    const ld ref = Gm[g][r] / (Mb[r] * Mb[r]);
+    for (int i = 0; i <= N; ++i) {
+      const ld h = fabsl(Gm[g][i]) / (Mb[i] * Mb[i]) / ref;
+      t->wh[g][i] = (double)h;
+      for (int j = 0; j < N; ++j) t->wc[g][i][j] = (double)(h * Eg[g][i][j]);
     }
   }
   // subcell averages (Fig. 1): N equal parts of each neighbour, troubled cell whole

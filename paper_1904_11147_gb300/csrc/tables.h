@@ -5,6 +5,12 @@
 // weights, smoothness-indicator quadratic forms, subcell averages).
 #pragma once
 
+#ifdef __CUDACC__
+#define DGT_HD __host__ __device__
+#else
+#define DGT_HD
+#endif
+
 namespace dgt {
 
 constexpr int kMaxN = 3;
@@ -31,11 +37,34 @@ struct Tabs {
   int neg[kMaxG];                            // point g has a negative linear weight
   double gpn[kMaxG][kMaxN + 1], gmn[kMaxG][kMaxN + 1]; // normalised split weights
   double sgp[kMaxG], sgm[kMaxG];                        // sigma+, sigma-
+  // The reconstruction of Steps 2-5 on the 2N differences d_k = avg[k+1] - avg[k] of
+  // neighbouring stencil averages (p_i - avg[N] and beta_i ignore constants), as the 2D
+  // limiters evaluate it.  With e = (d_i .. d_{i+N-1}) of stencil i, read from its far end
+  // for i <= N/2 and mirrored for the others, beta_i / M is a sum of squares,
+  //   N = 1: e_0^2;  N = 2: (e_0 + k e_1)^2 + o e_1^2;
+  //   N = 3: (e_0 + k e_1 + l e_2)^2 + m (e_1 + n e_2)^2 + o e_2^2,
+  // with the same constants for stencils i and N - i (class min(i, N - i)); the factors M go
+  // into the weights.  bform = {eps / M, o, m, k, l, n}.
+  double bform[2][6];
+  // p_i(x_g) - avg[N] = sum_j E_gij d_{i+j}.  With P_i proportional to the reciprocal of
+  // (eps / M + beta_i / M)^2: wh[g][i] = gamma_gi / M_i^2 over its value at the reference
+  // stencil weno_ref(N, g) and wc[g][i][j] = wh[g][i] E_gij, so that
+  //   u_g - avg[N] = sum_ij wc_gij P_i d_{i+j} / sum_i wh_gi P_i.
+  // At a point with one negative weight (sigma+ and sigma- of the split) wh and wc of that
+  // stencil are taken with |gamma|; qsp = {4 sigma+ - sigma- - 1, 4 sigma- - sigma+ + 1}.
+  double wh[kMaxG][kMaxN + 1], wc[kMaxG][kMaxN + 1][kMaxN], qsp[2];
   // initial projection: (N+4)-point Gauss rule
   int QP;
   double px[kMaxQ], pw[kMaxQ], ppsi[kMaxQ][kMaxN + 1];
   double gam_resid;                          // residual of the full Eq. (8) system
 };
+
+// Stencil whose weight is 1 in wh, and the stencil with a negative linear weight of the
+// CSWENO P3 rule at its inner points (-1: none).
+DGT_HD constexpr int weno_ref(int N, int g) { return N == 3 && g == 1 ? 2 : 1; }
+DGT_HD constexpr int weno_neg(int N, int g, bool parent) {
+  return N == 3 && !parent && g == 1 ? 3 : (N == 3 && !parent && g == 2 ? 0 : -1);
+}
 
 // Fills t for degree N; returns 0 on success.  parent: the limiter tables of the parent
 // WENO limiter (whole cells j-N .. j+N) instead of CSWENO's subcells.
