@@ -931,7 +931,7 @@ def dmr_arm(args, dist, rank, world, torch, dgl):
 def kernel_hash():
     import hashlib
     h = hashlib.sha1()
-    for f in ("dg_kernels2d.cu", "dg_common.cuh", "dg_shared.cuh"):
+    for f in ("dg_stage2.cu", "dg_weno.cuh", "dg_common.cuh", "dg_shared.cuh"):
         h.update(open(os.path.join(ROOT, "paper_1904_11147_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:12]
 

@@ -20,6 +20,10 @@ namespace dg {
 cudaError_t upload_tables1(const dgt::Tabs* tabs);
 cudaError_t upload_tables2(const dgt::Tabs* tabs);
 cudaError_t prepare2(int pde, int N);
+cudaError_t upload_tables_stage2(const dgt::Tabs* tabs);
+cudaError_t prepare_stage2_split(int pde, int N);
+int face_chunk2();
+int cell_chunk2();
 int tile_w1();
 int tile_w2();
 int tile_h2();
@@ -140,6 +144,7 @@ dg_status dg_ensure_tables_internal() {
   CK(upload_tables2(g_tabs));
   CK(upload_tables_parent(g_ptabs));
   CK(upload_tables_lim2(g_tabs, g_ptabs));
+  CK(upload_tables_stage2(g_tabs));
   done.push_back(dev);
   g_tables_dev = dev;
   return DG_OK;
@@ -181,8 +186,8 @@ struct dg_mesh {
   bool stage_split = false;
   double* fbuf = nullptr;
   long long fxt = 0, fyt = 0;
-  Tile* d_face_tiles = nullptr;
-  int n_face_tiles = 0;
+  Tile *d_face_tiles = nullptr, *d_cell_chunks = nullptr;
+  int n_face_tiles = 0, n_cell_chunks = 0;
   long long launches = 0;
   // CUDA graph of one full step
   cudaGraphExec_t gexec = nullptr;
@@ -243,6 +248,7 @@ extern "C" dg_status dg_mesh_destroy(dg_mesh* m) {
   cudaFree(m->d_lq);
   cudaFree(m->fbuf);
   cudaFree(m->d_face_tiles);
+  cudaFree(m->d_cell_chunks);
   cudaFree(m->d_cell_inst);
   for (auto& p : m->U) cudaFree(p);
   cudaFree(m->lim);
@@ -367,6 +373,8 @@ extern "C" dg_status dg_mesh_create(int dim, int pde, int N, int n_inst, const i
     I.xL = xL;
     I.yL = dim == 2 ? yL : 0.0;
     I.dt = 0.0;
+    I.sx = 2.0 / I.hx;
+    I.sy = 2.0 / I.hy;
     I.fx = fxoff;
     I.fy = fyoff;
     fxoff += (long long)(I.nx + 1) * I.ny;
@@ -462,6 +470,7 @@ extern "C" dg_status dg_mesh_create(int dim, int pde, int N, int n_inst, const i
   if (tv) m->stage_persistent = tv->persistent;
   if (dim == 2) {
     e = prepare2(pde, N);
+    if (e == cudaSuccess) e = prepare_stage2_split(pde, N);
     if (e == cudaSuccess) e = cudaMalloc(&m->d_queue, sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&m->d_lq, sizeof(unsigned int));
     if (e == cudaSuccess) e = build_stage_tiles(m, tv && tv->stage_ty ? tv->stage_ty : 8);
@@ -469,30 +478,35 @@ extern "C" dg_status dg_mesh_create(int dim, int pde, int N, int n_inst, const i
       dg_mesh_destroy(m);
       return fail(DG_ECUDA, "stage kernel set-up: %s", cudaGetErrorString(e));
     }
-    // split stage: face planes and face tiles (32 faces x 4 rows); without the memory the
-    // mesh keeps the fused stage
-    std::vector<Tile> ft;
+    // split stage: face planes, and chunks of every instance's face and cell index; without
+    // the memory the mesh keeps the fused stage
+    std::vector<Tile> ft, ct;
+    const long long fc = face_chunk2(), cc = cell_chunk2();
     for (int i = 0; i < n_inst; ++i) {
       const Inst& I = m->h_inst[i];
-      for (int y0 = 0; y0 < I.ny; y0 += 4)
-        for (int x0 = 0; x0 <= I.nx; x0 += 32) ft.push_back(Tile{i, x0, y0, 0});
-      for (int y0 = 0; y0 <= I.ny; y0 += 4)
-        for (int x0 = 0; x0 < I.nx; x0 += 32) ft.push_back(Tile{i, x0, y0, 1});
+      const long long nfx = (long long)(I.nx + 1) * I.ny, nfy = (long long)I.nx * (I.ny + 1), nc = (long long)I.nx * I.ny;
+      for (int k = 0; k * fc < nfx; ++k) ft.push_back(Tile{i, k, 0, 0});
+      for (int k = 0; k * fc < nfy; ++k) ft.push_back(Tile{i, k, 0, 1});
+      for (int k = 0; k * cc < nc; ++k) ct.push_back(Tile{i, k, 0, 0});
     }
     m->fxt = (fxoff + 31) / 32 * 32;
     m->fyt = (fyoff + 31) / 32 * 32;
     const size_t fbytes = sizeof(double) * (size_t)(m->N + 1) * m->V * (size_t)(m->fxt + m->fyt);
     if (cudaMalloc(&m->fbuf, fbytes) == cudaSuccess &&
         cudaMalloc(&m->d_face_tiles, sizeof(Tile) * ft.size()) == cudaSuccess &&
-        cudaMemcpy(m->d_face_tiles, ft.data(), sizeof(Tile) * ft.size(), cudaMemcpyHostToDevice) == cudaSuccess) {
+        cudaMemcpy(m->d_face_tiles, ft.data(), sizeof(Tile) * ft.size(), cudaMemcpyHostToDevice) == cudaSuccess &&
+        cudaMalloc(&m->d_cell_chunks, sizeof(Tile) * ct.size()) == cudaSuccess &&
+        cudaMemcpy(m->d_cell_chunks, ct.data(), sizeof(Tile) * ct.size(), cudaMemcpyHostToDevice) == cudaSuccess) {
       m->n_face_tiles = (int)ft.size();
+      m->n_cell_chunks = (int)ct.size();
       m->stage_split = !tv || tv->stage_ty == 0;
     } else {
       cudaGetLastError();
       cudaFree(m->fbuf);
       cudaFree(m->d_face_tiles);
+      cudaFree(m->d_cell_chunks);
       m->fbuf = nullptr;
-      m->d_face_tiles = nullptr;
+      m->d_face_tiles = m->d_cell_chunks = nullptr;
       m->stage_split = false;
     }
     if (bc == DG_BC_DMR && !m->fbuf) {
@@ -552,13 +566,18 @@ static __global__ void k_stage_time(double* __restrict__ bcd, const Inst* __rest
   }
 }
 
+static void k_stage_split(dg_mesh* m, int stage, int in, int out, double dt_all) {
+  LaunchArgs a = args<LaunchArgs>(m, 0, in, out);
+  a.tiles = m->d_cell_chunks;
+  a.ntiles = m->n_cell_chunks;
+  double* fy = m->fbuf + (size_t)(m->N + 1) * m->V * m->fxt;
+  launch_stage2_split(m->pde, m->N, a, stage, dt_all, m->d_face_tiles, m->n_face_tiles, m->fbuf, m->fxt, fy, m->fyt);
+}
+
 static void k_stage(dg_mesh* m, int stage, int in, int out, double dt_all) {
   if (m->bc == DG_BC_DMR) {
     // the stage evaluates L at the time of its input state (bcd), then the times advance
-    LaunchArgs a = args<LaunchArgs>(m, 0, in, out);
-    double* fy = m->fbuf + (size_t)(m->N + 1) * m->V * m->fxt;
-    launch_stage2_split(m->pde, m->N, a, stage, dt_all, m->d_face_tiles, m->n_face_tiles, m->fbuf, m->fxt, fy,
-                        m->fyt);
+    k_stage_split(m, stage, in, out, dt_all);
     k_stage_time<<<1, 32, 0, m->st>>>(m->d_bcd, m->d_inst, m->n_inst, stage, dt_all);
     m->launches += 3;
     return;
@@ -568,9 +587,7 @@ static void k_stage(dg_mesh* m, int stage, int in, int out, double dt_all) {
   } else {
     LaunchArgs a = args<LaunchArgs>(m, 0, in, out);
     if (m->stage_split) {
-      double* fy = m->fbuf + (size_t)(m->N + 1) * m->V * m->fxt;
-      launch_stage2_split(m->pde, m->N, a, stage, dt_all, m->d_face_tiles, m->n_face_tiles, m->fbuf, m->fxt, fy,
-                          m->fyt);
+      k_stage_split(m, stage, in, out, dt_all);
       m->launches += 2;
       return;
     }

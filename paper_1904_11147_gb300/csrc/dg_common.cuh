@@ -34,10 +34,12 @@ struct Inst {
   double xL, yL;  // lower-left corner
   double dt;      // per-instance time step (dg_set_dt)
   long long fx, fy;  // first x face / y face of the instance in the 2D face planes
+  double sx, sy;     // 2 / hx, 2 / hy
 };
 
 // A tile of the 2D stage / flag kernels: instance and lower-left cell of the tile.  The
-// face tiles of the split stage use `pad` for the face direction (0: x faces, 1: y faces).
+// split stage's tiles are chunks of the instance's face or cell index: x0 is the chunk's
+// number, `pad` the face direction (0: x faces, 1: y faces).
 struct Tile {
   int inst, x0, y0, pad;
 };
@@ -166,21 +168,6 @@ __device__ __forceinline__ void llf(int dir, const double* uL, const double* uR,
   const double a = nan_lr ? aL + aR : fmax(aL, aR);
 #pragma unroll
   for (int v = 0; v < V; ++v) fs[v] = inv_h * fma(-a, uR[v] - uL[v], fL[v] + fR[v]);
-}
-
-// The same flux without the 1/h factor: fs = (fL + fR) - alpha (uR - uL) = 2 f*.
-template <int DIM, int PDE>
-__device__ __forceinline__ void llf_sum(int dir, const double* uL, const double* uR, double* fs, double gam,
-                                        double gm1) {
-  constexpr int V = Phys<DIM, PDE>::V;
-  double fL[V], fR[V], aL, aR;
-  Phys<DIM, PDE>::flux(dir, uL, fL, aL, gam, gm1);
-  Phys<DIM, PDE>::flux(dir, uR, fR, aR, gam, gm1);
-  constexpr unsigned long long kAbs = 0x7fffffffffffffffull, kInf = 0x7ff0000000000000ull;
-  const bool nan_lr = ((__double_as_longlong(aL) & kAbs) > kInf) | ((__double_as_longlong(aR) & kAbs) > kInf);
-  const double a = nan_lr ? aL + aR : fmax(aL, aR);
-#pragma unroll
-  for (int v = 0; v < V; ++v) fs[v] = fma(-a, uR[v] - uL[v], fL[v] + fR[v]);
 }
 
 }  // namespace dg

@@ -1,11 +1,7 @@
 // 2D kernels (Cartesian cells, total-degree P^N, N = 1..3; Burgers V = 1, Euler V = 4).
 //
-//   k_face2     split stage, face pass: traces of the two cells, local Lax-Friedrichs
-//               flux at the face points, projection on the transverse modes (per face)
-//   k_cell2     split stage, cell pass: volume quadrature, lifting of the four faces,
-//               stage combination (per cell); the default form of one stage of Eq. (5)
-//   k_stage2    the same stage fused in one kernel per tile (halo warps, shared faces),
-//               an autotuner alternative
+//   k_stage2    one stage of Eq. (5) fused in one kernel per tile (halo warps, shared
+//               faces), an autotuner alternative to the split stage (dg_stage2.cu)
 //   k_flag2     TVB minmod indicator + ballot/scan compaction of troubled cells
 //   k_project2  initial L2 projection (Eq. (2))
 //   k_speed2    largest characteristic speed over the cell means
@@ -31,9 +27,7 @@ struct Lay {
   static constexpr int SIZE_DG = 3 * Q * Q * NP + N1 + 2 * Q * N1;
   static constexpr int SIZE_FLAG = 4 * NP + 1;
   static constexpr int SIZE_PROJ = 3 * 8 + 8 * N1;
-  static constexpr int SIZE_SPLIT = Q * N1;
-  static constexpr int SIZE_K = Q * N1 + N1;
-  static constexpr int SIZE = SIZE_DG + SIZE_FLAG + SIZE_PROJ + SIZE_SPLIT + SIZE_K;
+  static constexpr int SIZE = SIZE_DG + SIZE_FLAG + SIZE_PROJ;
 };
 __host__ __device__ constexpr int base_of(int N) {
   return N == 1 ? 0 : (N == 2 ? Lay<1>::SIZE : Lay<1>::SIZE + Lay<2>::SIZE);
@@ -57,10 +51,7 @@ struct Off {
   static constexpr int PW = PX + 8;              // [8]
   static constexpr int PQP = PW + 8;             // [8] (count in slot 0)
   static constexpr int PP = PQP + 8;             // [8][N1]
-  static constexpr int WDQ = PP + 8 * N1;        // [Q][N1] w_q psi_n'(x_q)
-  static constexpr int KQ = WDQ + Q * N1;        // [Q][N1] sqrt(2) psi_n(x_q) = psi_n(x_q) / psi_0
-  static constexpr int KP1 = KQ + Q * N1;        // [N1] sqrt(2) psi_n(1)
-  static constexpr int END = KP1 + N1;
+  static constexpr int END = PP + 8 * N1;
 };
 static_assert(Off<3>::END == Lay<1>::SIZE + Lay<2>::SIZE + Lay<3>::SIZE, "table layout");
 constexpr int kTabSize = Off<3>::END;
@@ -102,11 +93,6 @@ void pack(const dgt::Tabs& t, double* h) {
     for (int n = 0; n < N1; ++n) h[O::PP + q * N1 + n] = t.ppsi[q][n];
   }
   h[O::PQP] = t.QP;
-  for (int q = 0; q < Q; ++q)
-    for (int n = 0; n < N1; ++n) h[O::WDQ + q * N1 + n] = t.gw[q] * t.dpsi_q[q][n];
-  for (int q = 0; q < Q; ++q)
-    for (int n = 0; n < N1; ++n) h[O::KQ + q * N1 + n] = t.kq[q][n];
-  for (int n = 0; n < N1; ++n) h[O::KP1 + n] = t.kp1[n];
 }
 
 // ----------------------------------------------------------------------------- loads
@@ -133,35 +119,6 @@ __device__ __forceinline__ void load_cell(const double* __restrict__ U, long lon
     for (int m = 0; m < NP; ++m) {
       double x = __ldg(U + (long long)(v * NP + m) * ctot + g);
       bool flip = (fx && (mode_a(m) & 1)) != (fy && (mode_b(m) & 1));
-      u[v][m] = neg_if(x, flip);
-    }
-}
-
-// load_cell with the kBcDmr ghosts (dmr_ghost) for cells outside instance `inst`.
-// t: the time of the state U.
-template <int V, int NP>
-__device__ __forceinline__ void load_cell_bc(const double* __restrict__ U, long long ctot, const Inst& I, int inst,
-                                             int ix, int iy, int bc, const double* __restrict__ bcd, double t,
-                                             double (&u)[V][NP]) {
-  if (bc != kBcDmr || (ix >= 0 && ix < I.nx && iy >= 0 && iy < I.ny)) {
-    load_cell<V, NP>(U, ctot, I, ix, iy, bc, u);
-    return;
-  }
-  const Ghost gh = dmr_ghost(I, inst, ix, iy, bcd, t);
-  if (gh.c) {  // constant state: U_00 = mean / psi_0^2 = 2 mean, no other mode
-#pragma unroll
-    for (int v = 0; v < V; ++v)
-#pragma unroll
-      for (int m = 0; m < NP; ++m) u[v][m] = m == 0 ? 2.0 * gh.c[v] : 0.0;
-    return;
-  }
-  const long long g = I.off + (long long)gh.jy * I.nx + gh.jx;
-#pragma unroll
-  for (int v = 0; v < V; ++v)
-#pragma unroll
-    for (int m = 0; m < NP; ++m) {
-      const double x = __ldg(U + (long long)(v * NP + m) * ctot + g);
-      const bool flip = ((gh.fx && (mode_a(m) & 1)) != (gh.fy && (mode_b(m) & 1))) != (gh.fv && v == 2);
       u[v][m] = neg_if(x, flip);
     }
 }
@@ -504,464 +461,6 @@ __global__ void __launch_bounds__((TYS + 3) * 32, 1)
 #undef sE
 #undef sN
 
-// ----------------------------------------------------------------------------- split stage
-// The same stage of Eq. (5) as two passes without block barriers or halo work:
-//   k_face2  one thread per face: the traces of the two cells at the Q face points, the
-//            local Lax-Friedrichs flux there, and its projection onto the transverse modes
-//              P_b = sum_q w_q psi_b(s_q) [f(uL) + f(uR) - alpha (uR - uL)],  b = 0..N,
-//            stored in planes [v*(N+1) + b][face] (x faces and y faces apart); the traces
-//            are formed doubled (face_trace2), so the planes hold 2^d P_b, d the degree
-//            of homogeneity of the flux (1 Euler, 2 Burgers);
-//   k_cell2  one thread per cell: the volume term (at doubled point values, likewise),
-//            the lifting of the four faces' P_b and the stage combination, with 2^-d
-//            folded into the scalings 2/h and 1/h.
-// Every face flux is computed once; all lanes of every warp do the same work.
-
-// Values at the Q Gauss points of sum_t e_t psi_t(s).  The points are symmetric
-// (s_{Q-1-q} = -s_q) and psi_t has the parity of t, so the even and odd sums are formed
-// once per pair of points; psi_0 is constant.
-template <int N>
-__device__ __forceinline__ void eval_gauss(const double (&e)[N + 1], double (&out)[N + 1]) {
-  using O = Off<N>;
-  constexpr int Q = N + 1;
-  const double p0 = e[0] * T(O::PQ);
-#pragma unroll
-  for (int q = 0; q < Q / 2; ++q) {
-    double ev = p0, od = e[1] * T(O::PQ + q * (N + 1) + 1);
-#pragma unroll
-    for (int t = 2; t <= N; ++t) {
-      if (t & 1) od = fma(e[t], T(O::PQ + q * (N + 1) + t), od);
-      else ev = fma(e[t], T(O::PQ + q * (N + 1) + t), ev);
-    }
-    out[q] = ev + od;
-    out[Q - 1 - q] = ev - od;
-  }
-  if constexpr (Q & 1) {
-    double ev = p0;
-#pragma unroll
-    for (int t = 2; t <= N; t += 2) ev = fma(e[t], T(O::PQ + (Q / 2) * (N + 1) + t), ev);
-    out[Q / 2] = ev;
-  }
-}
-
-// Twice the values at the Q Gauss points of sum_t e_t psi_t(s) / psi_0 (e given over
-// psi_0): 2 sum_t (e_t / psi_0) psi_t(s) psi_0 = e_0 + sum_{t>=1} e_t sqrt(2) psi_t(s), so the
-// constant term enters without a multiplication.  Symmetric pairs as in eval_gauss.
-template <int N>
-__device__ __forceinline__ void eval_gauss2(const double (&e)[N + 1], double (&out)[N + 1]) {
-  using O = Off<N>;
-  constexpr int Q = N + 1;
-#pragma unroll
-  for (int q = 0; q < Q / 2; ++q) {
-    double ev = e[0], od = e[1] * T(O::KQ + q * (N + 1) + 1);
-#pragma unroll
-    for (int t = 2; t <= N; ++t) {
-      if (t & 1) od = fma(e[t], T(O::KQ + q * (N + 1) + t), od);
-      else ev = fma(e[t], T(O::KQ + q * (N + 1) + t), ev);
-    }
-    out[q] = ev + od;
-    out[Q - 1 - q] = ev - od;
-  }
-  if constexpr (Q & 1) {
-    double ev = e[0];
-#pragma unroll
-    for (int t = 2; t <= N; t += 2) ev = fma(e[t], T(O::KQ + (Q / 2) * (N + 1) + t), ev);
-    out[Q / 2] = ev;
-  }
-}
-
-// Twice the trace of a cell on its face normal to `dir` at the Q face points, the +1 side
-// (east / north) or, with minus = true, the -1 side (west / south), whose normal modes of
-// odd degree enter with the opposite sign.  With psi_n(1) = psi_0 sqrt(2 n + 1), the sum
-// over the normal degree is formed over psi_0 (its constant term needs no multiplication)
-// and eval_gauss2 doubles the result; the fluxes of the split stage are homogeneous in the
-// state (Euler of degree 1, Burgers of degree 2), so the passes carry the factor 2 and
-// remove it, exactly, in the final scalings.  The mirror image of a cell (outflow ghost)
-// gives a bitwise identical trace on the shared face.
-template <int N, int V, int NP>
-__device__ __forceinline__ void face_trace2(const double (&u)[V][NP], int dir, bool minus, double (&tr)[N + 1][V]) {
-  using O = Off<N>;
-#pragma unroll
-  for (int v = 0; v < V; ++v) {
-    double e[N + 1], val[N + 1];
-#pragma unroll
-    for (int t = 0; t <= N; ++t) {  // transverse degree t, normal degree n
-      double s = u[v][dir == 0 ? mode_idx(0, t) : mode_idx(t, 0)];
-#pragma unroll
-      for (int n = 1; n <= N - t; ++n) {
-        const double x = u[v][dir == 0 ? mode_idx(n, t) : mode_idx(t, n)];
-        s = fma(neg_if(x, minus && (n & 1)), T(O::KP1 + n), s);
-      }
-      e[t] = s;
-    }
-    eval_gauss2<N>(e, val);
-#pragma unroll
-    for (int q = 0; q <= N; ++q) tr[q][v] = val[q];
-  }
-}
-
-// Trace of a cell on its face normal to `dir` at the Q face points: the +1 side
-// (east / north) or, with minus = true, the -1 side (west / south), whose normal modes of
-// odd degree enter with the opposite sign.  The mirror image of a cell (outflow ghost)
-// therefore gives a bitwise identical trace on the shared face.
-template <int N, int V, int NP>
-__device__ __forceinline__ void face_trace(const double (&u)[V][NP], int dir, bool minus, double (&tr)[N + 1][V]) {
-  using O = Off<N>;
-#pragma unroll
-  for (int v = 0; v < V; ++v) {
-    double e[N + 1], val[N + 1];
-#pragma unroll
-    for (int t = 0; t <= N; ++t) {  // transverse degree t, normal degree n
-      double s = u[v][dir == 0 ? mode_idx(0, t) : mode_idx(t, 0)] * T(O::P1);
-#pragma unroll
-      for (int n = 1; n <= N - t; ++n) {
-        const double x = u[v][dir == 0 ? mode_idx(n, t) : mode_idx(t, n)];
-        s = fma(neg_if(x, minus && (n & 1)), T(O::P1 + n), s);
-      }
-      e[t] = s;
-    }
-    eval_gauss<N>(e, val);
-#pragma unroll
-    for (int q = 0; q <= N; ++q) tr[q][v] = val[q];
-  }
-}
-
-// Face tiles: 32 faces along x by 4 rows; Tile::pad = 0 for x faces (k = 0..nx, j < ny),
-// 1 for y faces (k < nx, j = 0..ny).  Face k of a row lies between cells k-1 and k.
-template <int PDE, int N>
-__global__ void __launch_bounds__(128) k_face2(const double* __restrict__ us, const Inst* __restrict__ insts,
-                                               const Tile* __restrict__ tiles, long long ctot, int bc, double gam,
-                                               double* __restrict__ fx, long long fxt, double* __restrict__ fy,
-                                               long long fyt, const double* __restrict__ bcd, int stage,
-                                               double dt_all) {
-  using O = Off<N>;
-  constexpr int V = nv_of(2, PDE), NP = np_of(2, N), Q = N + 1;
-  const Tile tile = tiles[blockIdx.x];
-  const Inst I = insts[tile.inst];
-  const int dir = tile.pad;
-  const int k = tile.x0 + (threadIdx.x & 31), j = tile.y0 + (threadIdx.x >> 5);
-  if (dir == 0 ? (k > I.nx || j >= I.ny) : (k >= I.nx || j > I.ny)) return;
-  const double gm1 = gam - 1.0;
-  // kBcDmr: the stage's input holds at t^n, t^n + dt, t^n + dt/2 for stages 1, 2, 3
-  double t_in = 0.0;
-  if (bc == kBcDmr) t_in = dmr_time(bcd, tile.inst, 2) + (stage == 1 ? 0.0 : (stage == 2 ? 1.0 : 0.5)) * (dt_all > 0.0 ? dt_all : I.dt);
-  double tL[Q][V], tR[Q][V];
-  {
-    double u[V][NP];
-    load_cell_bc<V, NP>(us, ctot, I, tile.inst, dir == 0 ? k - 1 : k, dir == 0 ? j : j - 1, bc, bcd, t_in, u);
-    face_trace2<N>(u, dir, false, tL);
-  }
-  {
-    double u[V][NP];
-    load_cell_bc<V, NP>(us, ctot, I, tile.inst, k, j, bc, bcd, t_in, u);
-    face_trace2<N>(u, dir, true, tR);
-  }
-  double G[Q][V];
-#pragma unroll
-  for (int q = 0; q < Q; ++q) llf_sum<2, PDE>(dir, tL[q], tR[q], G[q], gam, gm1);
-  // P_b = sum_q w_q psi_b(s_q) G(q), summed over symmetric pairs of points
-  double* const base = dir == 0 ? fx + I.fx + (long long)j * (I.nx + 1) + k : fy + I.fy + (long long)j * I.nx + k;
-  const long long stride = dir == 0 ? fxt : fyt;
-#pragma unroll
-  for (int v = 0; v < V; ++v) {
-    double S[Q / 2 + 1], D[Q / 2 + 1];
-#pragma unroll
-    for (int q = 0; q < Q / 2; ++q) {
-      S[q] = G[q][v] + G[Q - 1 - q][v];
-      D[q] = G[q][v] - G[Q - 1 - q][v];
-    }
-#pragma unroll
-    for (int b = 0; b <= N; ++b) {
-      double P = 0.0;
-      bool first = true;
-#pragma unroll
-      for (int q = 0; q < Q / 2; ++q) {
-        const double x = (b & 1) ? D[q] : S[q];
-        P = first ? x * T(O::WPQ + q * (N + 1) + b) : fma(x, T(O::WPQ + q * (N + 1) + b), P);
-        first = false;
-      }
-      if ((Q & 1) && !(b & 1)) P = fma(G[Q / 2][v], T(O::WPQ + (Q / 2) * (N + 1) + b), P);
-      base[(long long)(v * (N + 1) + b) * stride] = P;
-    }
-  }
-}
-
-// One thread per cell over the 32 x 8 cell tiles (lane = column, warp = row).
-// Two blocks per SM (at most 128 registers) except for Euler P3, which needs more registers.
-template <int PDE, int N>
-__global__ void __launch_bounds__(256, (PDE == 1 && N == 3) ? 1 : 2) k_cell2(const double* __restrict__ un, const double* __restrict__ us,
-                                               double* __restrict__ out, const Inst* __restrict__ insts,
-                                               const Tile* __restrict__ tiles, long long ctot, int stage,
-                                               double dt_all, const double* __restrict__ fx, long long fxt,
-                                               const double* __restrict__ fy, long long fyt, double gam) {
-  using O = Off<N>;
-  constexpr int V = nv_of(2, PDE), NP = np_of(2, N), Q = N + 1;
-  const Tile tile = tiles[blockIdx.x];
-  const Inst I = insts[tile.inst];
-  const int ix = tile.x0 + (threadIdx.x & 31), iy = tile.y0 + (threadIdx.x >> 5);
-  if (ix >= I.nx || iy >= I.ny) return;
-  const long long g = I.off + (long long)iy * I.nx + ix;
-  const double gm1 = gam - 1.0, hgm1 = -0.5 * gm1;
-  // Euler P3 keeps the cell's modes in shared memory (one slot per thread and mode: no
-  // sharing, no barrier), which leaves the registers to the sum factorisation
-  constexpr bool kSmemU = PDE == 1 && N == 3;
-  extern __shared__ double s_u[];
-  double u[V][NP];
-#pragma unroll
-  for (int v = 0; v < V; ++v)
-#pragma unroll
-    for (int m = 0; m < NP; ++m) {
-      const double x = __ldg(us + (long long)(v * NP + m) * ctot + g);
-      if constexpr (kSmemU) s_u[(v * NP + m) * 256 + threadIdx.x] = x;
-      else u[v][m] = x;
-    }
-  // volume term, unscaled: X_ab = sum_q w w f psi_a' psi_b (a >= 1), Y_ab likewise with g (b >= 1),
-  // sum-factorised: for every x point the column sums over y, then the x weights
-  double X[V][NP], Y[V][NP];
-#pragma unroll
-  for (int v = 0; v < V; ++v)
-#pragma unroll
-    for (int m = 0; m < NP; ++m) X[v][m] = Y[v][m] = 0.0;
-  if constexpr (kSmemU) {
-#pragma unroll
-    for (int qx = 0; qx < Q; ++qx) {
-      double tb[V][N + 1];
-#pragma unroll
-      for (int v = 0; v < V; ++v)
-#pragma unroll
-        for (int b = 0; b <= N; ++b) {
-          // t_b over psi_0 (see eval_gauss2): the constant term needs no multiplication
-          double t = s_u[(v * NP + mode_idx(0, b)) * 256 + threadIdx.x];
-#pragma unroll
-          for (int a = 1; a <= N - b; ++a)
-            t = fma(s_u[(v * NP + mode_idx(a, b)) * 256 + threadIdx.x], T(O::KQ + qx * (N + 1) + a), t);
-          tb[v][b] = t;
-        }
-      double col[V][Q];  // twice u at (x_qx, y_qy)
-#pragma unroll
-      for (int v = 0; v < V; ++v) {
-        double val[Q];
-        eval_gauss2<N>(tb[v], val);
-#pragma unroll
-        for (int qy = 0; qy < Q; ++qy) col[v][qy] = val[qy];
-      }
-      // column sums over symmetric pairs of y points: G_b = sum_y w psi_b(y) f (b < N),
-      // H_b = sum_y w psi_b'(y) g (b >= 1), stored at H[b - 1]; Q = N + 1 is even here
-      static_assert((Q & 1) == 0, "P3: no middle point");
-      double G[V][N], H[V][N];
-#pragma unroll
-      for (int qp = 0; qp < Q / 2; ++qp) {
-        double fA[V], gA[V], fB[V], gB[V];
-#pragma unroll
-        for (int side = 0; side < 2; ++side) {
-          const int qy = side == 0 ? qp : Q - 1 - qp;
-          const double rho = col[0][qy], mx = col[1][qy], my = col[2][qy], E = col[3][qy];
-          const double r = rcp_d(rho);
-          const double vx = mx * r, vy = my * r;
-          const double p = fma(hgm1, fma(mx, vx, my * vy), gm1 * E);  // (gamma-1)(E - rho |v|^2 / 2)
-          const double ep = E + p;
-          double* f = side == 0 ? fA : fB;
-          double* gg = side == 0 ? gA : gB;
-          f[0] = mx;
-          f[1] = fma(mx, vx, p);
-          f[2] = my * vx;
-          f[3] = ep * vx;
-          gg[0] = my;
-          gg[1] = f[2];
-          gg[2] = fma(my, vy, p);
-          gg[3] = ep * vy;
-        }
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-          const double fS = fA[v] + fB[v], fD = fA[v] - fB[v], gS = gA[v] + gB[v], gD = gA[v] - gB[v];
-#pragma unroll
-          for (int b = 0; b < N; ++b) {
-            const double x = (b & 1) ? fD : fS;
-            G[v][b] = qp == 0 ? x * T(O::WPQ + b) : fma(x, T(O::WPQ + qp * (N + 1) + b), G[v][b]);
-          }
-#pragma unroll
-          for (int b = 1; b <= N; ++b) {
-            const double x = (b & 1) ? gS : gD;
-            H[v][b - 1] = qp == 0 ? x * T(O::WDQ + b) : fma(x, T(O::WDQ + qp * (N + 1) + b), H[v][b - 1]);
-          }
-        }
-      }
-#pragma unroll
-      for (int v = 0; v < V; ++v) {
-#pragma unroll
-        for (int b = 0; b < N; ++b)
-#pragma unroll
-          for (int a = 1; a <= N - b; ++a)
-            X[v][mode_idx(a, b)] = fma(T(O::WDQ + qx * (N + 1) + a), G[v][b], X[v][mode_idx(a, b)]);
-#pragma unroll
-        for (int b = 1; b <= N; ++b)
-#pragma unroll
-          for (int a = 0; a <= N - b; ++a)
-            Y[v][mode_idx(a, b)] = fma(T(O::WPQ + qx * (N + 1) + a), H[v][b - 1], Y[v][mode_idx(a, b)]);
-      }
-    }
-  } else {
-    // x points in symmetric pairs (t_b formed once per pair).  Euler P3 takes the direct
-    // form (one quadrature point at a time), which needs fewer registers.
-    constexpr bool kPair = true;
-    constexpr int NX = (Q + 1) / 2;
-  #pragma unroll
-    for (int qp = 0; qp < NX; ++qp) {
-      // t_b(x) = sum_a U_ab psi_a(x) at the pair of points x_qp and x_{Q-1-qp} = -x_qp (parts
-      // even and odd in a), or at one point (for the middle point 0, psi_a vanishes for odd a)
-      const bool single = !kPair || ((Q & 1) && qp == Q / 2);
-      const bool zero = (Q & 1) && qp == Q / 2;
-      double tb[2][V][N + 1];
-  #pragma unroll
-      for (int v = 0; v < V; ++v)
-  #pragma unroll
-        for (int b = 0; b <= N; ++b) {
-          // over psi_0 (see eval_gauss2): the constant term needs no multiplication
-          double ev = u[v][mode_idx(0, b)], od = 0.0;
-  #pragma unroll
-          for (int a = 1; a <= N - b; ++a) {
-            if (a & 1) {
-              if (zero) continue;
-              if (single) ev = fma(u[v][mode_idx(a, b)], T(O::KQ + qp * (N + 1) + a), ev);
-              else od = a == 1 ? u[v][mode_idx(a, b)] * T(O::KQ + qp * (N + 1) + a)
-                               : fma(u[v][mode_idx(a, b)], T(O::KQ + qp * (N + 1) + a), od);
-            } else {
-              ev = fma(u[v][mode_idx(a, b)], T(O::KQ + qp * (N + 1) + a), ev);
-            }
-          }
-          const bool has_od = !single && b < N;
-          tb[0][v][b] = has_od ? ev + od : ev;
-          tb[1][v][b] = has_od ? ev - od : ev;
-        }
-  #pragma unroll
-      for (int side = 0; side < 2; ++side) {
-        if (single && side == 1) break;
-        const int qx = side == 0 ? qp : Q - 1 - qp;
-        const bool mid = (Q & 1) && qx == Q / 2;
-        double col[V][Q];  // twice u at (x_qx, y_qy) for every qy
-  #pragma unroll
-        for (int v = 0; v < V; ++v) {
-          double val[Q];
-          eval_gauss2<N>(tb[side][v], val);
-  #pragma unroll
-          for (int qy = 0; qy < Q; ++qy) col[v][qy] = val[qy];
-        }
-        double F[Q][V], Gq[Q][V];
-  #pragma unroll
-        for (int qy = 0; qy < Q; ++qy) {
-          if constexpr (PDE == 0) {
-            const double h = 0.5 * col[0][qy] * col[0][qy];
-            F[qy][0] = h;
-            Gq[qy][0] = h;
-          } else {
-            const double rho = col[0][qy], mx = col[1][qy], my = col[2][qy], E = col[3][qy];
-            const double r = rcp_d(rho);
-            const double vx = mx * r, vy = my * r;
-            const double p = fma(hgm1, fma(mx, vx, my * vy), gm1 * E);  // (gamma-1)(E - rho |v|^2 / 2)
-            const double ep = E + p;
-            F[qy][0] = mx;
-            F[qy][1] = fma(mx, vx, p);
-            F[qy][2] = my * vx;
-            F[qy][3] = ep * vx;
-            Gq[qy][0] = my;
-            Gq[qy][1] = F[qy][2];
-            Gq[qy][2] = fma(my, vy, p);
-            Gq[qy][3] = ep * vy;
-          }
-        }
-  #pragma unroll
-        for (int v = 0; v < V; ++v) {
-          // sums and differences over the symmetric pairs of y points
-          double fS[Q / 2 + 1], fD[Q / 2 + 1], gS[Q / 2 + 1], gD[Q / 2 + 1];
-  #pragma unroll
-          for (int q = 0; q < Q / 2; ++q) {
-            fS[q] = F[q][v] + F[Q - 1 - q][v];
-            fD[q] = F[q][v] - F[Q - 1 - q][v];
-            gS[q] = Gq[q][v] + Gq[Q - 1 - q][v];
-            gD[q] = Gq[q][v] - Gq[Q - 1 - q][v];
-          }
-          // x derivative part: G_b = sum_y w psi_b(y) f (psi_b has the parity of b)
-  #pragma unroll
-          for (int b = 0; b < N; ++b) {
-            double G = 0.0;
-  #pragma unroll
-            for (int q = 0; q < Q / 2; ++q)
-              G = q == 0 ? ((b & 1) ? fD[0] : fS[0]) * T(O::WPQ + b)
-                         : fma((b & 1) ? fD[q] : fS[q], T(O::WPQ + q * (N + 1) + b), G);
-            if ((Q & 1) && !(b & 1)) G = fma(F[Q / 2][v], T(O::WPQ + (Q / 2) * (N + 1) + b), G);
-  #pragma unroll
-            for (int a = 1; a <= N - b; ++a) {
-              if (mid && !(a & 1)) continue;  // psi_a'(0) = 0 for even a
-              X[v][mode_idx(a, b)] = fma(T(O::WDQ + qx * (N + 1) + a), G, X[v][mode_idx(a, b)]);
-            }
-          }
-          // y derivative part: H_b = sum_y w psi_b'(y) g (psi_b' has the parity of b + 1)
-  #pragma unroll
-          for (int b = 1; b <= N; ++b) {
-            double H = 0.0;
-  #pragma unroll
-            for (int q = 0; q < Q / 2; ++q)
-              H = q == 0 ? ((b & 1) ? gS[0] : gD[0]) * T(O::WDQ + b)
-                         : fma((b & 1) ? gS[q] : gD[q], T(O::WDQ + q * (N + 1) + b), H);
-            if ((Q & 1) && (b & 1)) H = fma(Gq[Q / 2][v], T(O::WDQ + (Q / 2) * (N + 1) + b), H);
-  #pragma unroll
-            for (int a = 0; a <= N - b; ++a) {
-              if (mid && (a & 1)) continue;  // psi_a(0) = 0 for odd a
-              Y[v][mode_idx(a, b)] = fma(T(O::WPQ + qx * (N + 1) + a), H, Y[v][mode_idx(a, b)]);
-            }
-          }
-        }
-      }
-    }
-  }
-  // acc = (2/hx) X + (2/hy) Y - (1/hx) psi_a(1) [P_b(E) -+ P_b(W)] - (1/hy) psi_b(1) [P_a(N) -+ P_a(S)],
-  // where X, Y and the P_b were formed from doubled states: the scalings take 2^-d (exact)
-  constexpr double kHom = PDE == 1 ? 0.5 : 0.25;
-  const double sx = (2.0 / I.hx) * kHom, sy = (2.0 / I.hy) * kHom, ihx = 0.5 * sx, ihy = 0.5 * sy;
-  double cx[N + 1], cy[N + 1];
-#pragma unroll
-  for (int n = 0; n <= N; ++n) {
-    cx[n] = -ihx * T(O::P1 + n);
-    cy[n] = -ihy * T(O::P1 + n);
-  }
-  const double* const pw = fx + I.fx + (long long)iy * (I.nx + 1) + ix;  // west face; east = pw + 1
-  const double* const ps = fy + I.fy + (long long)iy * I.nx + ix;        // south face; north = ps + nx
-  const double dt = dt_all > 0.0 ? dt_all : I.dt;
-#pragma unroll
-  for (int v = 0; v < V; ++v) {
-    double acc[NP];
-#pragma unroll
-    for (int m = 0; m < NP; ++m) {
-      const bool hx_ = mode_a(m) >= 1, hy_ = mode_b(m) >= 1;
-      acc[m] = hx_ ? (hy_ ? fma(sx, X[v][m], sy * Y[v][m]) : sx * X[v][m]) : (hy_ ? sy * Y[v][m] : 0.0);
-    }
-#pragma unroll
-    for (int b = 0; b <= N; ++b) {
-      const long long pl = (long long)(v * (N + 1) + b);
-      const double PW = __ldg(pw + pl * fxt), PE = __ldg(pw + pl * fxt + 1);
-      const double PS = __ldg(ps + pl * fyt), PN = __ldg(ps + pl * fyt + I.nx);
-      const double Dx = PE - PW, Sx = PE + PW, Dy = PN - PS, Sy = PN + PS;
-#pragma unroll
-      for (int a = 0; a <= N - b; ++a) {
-        const int mx = mode_idx(a, b);  // x faces: normal degree a, transverse degree b
-        acc[mx] = fma(cx[a], (a & 1) ? Sx : Dx, acc[mx]);
-        const int my = mode_idx(b, a);  // y faces: transverse degree b (in x), normal a
-        acc[my] = fma(cy[a], (a & 1) ? Sy : Dy, acc[my]);
-      }
-    }
-#pragma unroll
-    for (int m = 0; m < NP; ++m) {
-      const long long idx = (long long)(v * NP + m) * ctot + g;
-      const double e = fma(dt, acc[m], us[idx]);
-      double r;
-      if (stage == 1) r = e;
-      else if (stage == 2) r = fma(0.75, un[idx], 0.25 * e);
-      else r = fma(1.0 / 3.0, un[idx], (2.0 / 3.0) * e);
-      out[idx] = r;
-    }
-  }
-}
-
 // ----------------------------------------------------------------------------- indicator
 // TVB modified minmod (Cockburn-Shu) on conserved variables, x test on the east/west
 // edge midpoints and y test on the north/south ones.  The face values and means are
@@ -1166,11 +665,6 @@ static cudaError_t prep_stage2() {
   cudaError_t e = cudaFuncSetAttribute(k2::k_stage2<PDE, N, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)stage_smem2<PDE, N, 8>());
   if (e != cudaSuccess) return e;
-  if (PDE == 1 && N == 3) {
-    e = cudaFuncSetAttribute(k2::k_cell2<PDE, N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(sizeof(double) * 4 * 10 * 256));
-    if (e != cudaSuccess) return e;
-  }
   return cudaFuncSetAttribute(k2::k_stage2<PDE, N, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)stage_smem2<PDE, N, 4>());
 }
@@ -1186,20 +680,6 @@ static void run_stage2(const LaunchArgs& a, int stage, double dt_all, int* queue
   const size_t bytes = stage_smem2<PDE, N, TYS>();
   k2::k_stage2<PDE, N, TYS><<<queue ? grid : a.ntiles, (TYS + 3) * 32, bytes, a.st>>>(
       a.un, a.us, a.out, a.inst, a.tiles, a.ctot, a.bc, stage, dt_all, a.gam, a.ntiles, queue);
-}
-// dynamic shared memory of the cell pass: the modes of its 256 cells for Euler P3
-static constexpr size_t cell_smem2(int pde, int N) {
-  return pde == 1 && N == 3 ? sizeof(double) * 4 * 10 * 256 : 0;
-}
-
-// split form: the face pass over the face tiles, then the cell pass over the 32 x 8 cell tiles
-void launch_stage2_split(int pde, int N, const LaunchArgs& a, int stage, double dt_all, const Tile* face_tiles,
-                         int nface_tiles, double* fx, long long fxt, double* fy, long long fyt) {
-  DG_DISPATCH2(pde, N, (k2::k_face2<P_, N_><<<nface_tiles, 128, 0, a.st>>>(a.us, a.inst, face_tiles, a.ctot, a.bc,
-                                                                            a.gam, fx, fxt, fy, fyt, a.bcd, stage,
-                                                                            dt_all)));
-  DG_DISPATCH2(pde, N, (k2::k_cell2<P_, N_><<<a.ntiles, 256, cell_smem2(P_, N_), a.st>>>(a.un, a.us, a.out, a.inst, a.tiles, a.ctot,
-                                                                         stage, dt_all, fx, fxt, fy, fyt, a.gam)));
 }
 int tile_w2() { return k2::TX; }
 int tile_h2() { return k2::TY; }

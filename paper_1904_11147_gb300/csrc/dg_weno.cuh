@@ -21,6 +21,15 @@ struct Reg64 {  // the opaque constants 1.0 and -0.0
   __device__ __forceinline__ double mul(double x, double y) const { return fma(x, y, nz); }
 };
 
+// rcp_d with its constant in a register
+__device__ __forceinline__ double rcp_k(double x, const Reg64& K) {
+  if (((unsigned)__double2hiint(x) & 0x7fffffffu) - 0x00100000u >= 0x7fc00000u) return 1.0 / x;
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x, y, K.one);
+  return fma(y, fma(e, e, e), y);
+}
+
 // Tables of one limiter (degree N, CSWENO or parent) as the kernels keep them in shared memory.
 template <int N>
 struct LimTab {
