@@ -25,6 +25,10 @@ cudaError_t prepare_stage2_split(int pde, int N);
 int face_chunk2();
 int cell_chunk2();
 int tile_w1();
+int step_tile1();
+cudaError_t upload_tables_step1(const dgt::Tabs* tabs);
+cudaError_t prepare_step1(int pde, int N);
+void launch_step1(int pde, int N, const LaunchArgs& a, double M, unsigned long long* totals);
 int tile_w2();
 int tile_h2();
 void launch_stage1(int pde, int N, const LaunchArgs& a, int stage, double dt_all);
@@ -145,6 +149,7 @@ dg_status dg_ensure_tables_internal() {
   CK(upload_tables_parent(g_ptabs));
   CK(upload_tables_lim2(g_tabs, g_ptabs));
   CK(upload_tables_stage2(g_tabs));
+  CK(upload_tables_step1(g_tabs));
   done.push_back(dev);
   g_tables_dev = dev;
   return DG_OK;
@@ -181,6 +186,9 @@ struct dg_mesh {
   int stage_persistent = 0;  // persistent tile queue (1) or one block per tile (0)
   int* d_queue = nullptr;
   unsigned int* d_lq = nullptr;  // work counter of the 2D Euler limiter
+  // 1D: tiles of the whole-step kernel
+  Tile* d_step_tiles = nullptr;
+  int n_step_tiles = 0;
   // split 2D stage (face pass + cell pass; stage_ty == 0): face flux planes, x faces then
   // y faces, with their plane strides, and the face tiles
   bool stage_split = false;
@@ -244,6 +252,7 @@ extern "C" dg_status dg_mesh_destroy(dg_mesh* m) {
   cudaFree(m->d_inst);
   cudaFree(m->d_tiles);
   cudaFree(m->d_stage_tiles);
+  cudaFree(m->d_step_tiles);
   cudaFree(m->d_queue);
   cudaFree(m->d_lq);
   cudaFree(m->fbuf);
@@ -468,6 +477,20 @@ extern "C" dg_status dg_mesh_create(int dim, int pde, int N, int n_inst, const i
   const TuneVal* tv = tune_find(TuneKey{dim, pde, N, size_class(off)});
   if (tv) m->limit_blocks = m->sms * tv->limit_per_sm;
   if (tv) m->stage_persistent = tv->persistent;
+  if (dim == 1) {
+    std::vector<Tile> st;
+    const long long tw = step_tile1();
+    for (int i = 0; i < n_inst; ++i)
+      for (int k = 0; k * tw < m->h_inst[i].nx; ++k) st.push_back(Tile{i, k, 0, 0});
+    m->n_step_tiles = (int)st.size();
+    e = prepare_step1(pde, N);
+    if (e == cudaSuccess) e = cudaMalloc(&m->d_step_tiles, sizeof(Tile) * st.size());
+    if (e == cudaSuccess) e = cudaMemcpy(m->d_step_tiles, st.data(), sizeof(Tile) * st.size(), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) {
+      dg_mesh_destroy(m);
+      return fail(DG_ECUDA, "step kernel set-up: %s", cudaGetErrorString(e));
+    }
+  }
   if (dim == 2) {
     e = prepare2(pde, N);
     if (e == cudaSuccess) e = prepare_stage2_split(pde, N);
@@ -1073,6 +1096,31 @@ extern "C" dg_status dg_step(dg_mesh* m, double dt, int indicator, double tvb_M)
     if (s != DG_OK) return s;
   }
   m->cur = 0;
+  if (m->dim == 1 && indicator == DG_IND_TVB && m->limiter == DG_LIM_CSWENO && !m->pp_on) {
+    // the whole step in one kernel, u^n to the next buffer; the buffers then change places.
+    // Inside a caller's stream capture the recorded work must not depend on the replay's
+    // number: there the result is copied back instead.
+    LaunchArgs a = args<LaunchArgs>(m, 0, 0, 1);
+    a.tiles = m->d_step_tiles;
+    a.ntiles = m->n_step_tiles;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (m->st) CK(cudaStreamIsCapturing(m->st, &cs));
+    launch_step1(m->pde, m->N, a, tvb_M, m->flag_totals);
+    CK(cudaGetLastError());
+    m->launches++;
+    if (cs != cudaStreamCaptureStatusNone) {
+      CK(cudaMemcpyAsync(m->U[0], m->U[1], sizeof(double) * m->ctot * m->V * m->NP, cudaMemcpyDeviceToDevice, m->st));
+    } else {
+      std::swap(m->U[0], m->U[1]);
+      if (m->gexec) {  // a graph of another kind of step holds the buffers' old places
+        cudaGraphExecDestroy(m->gexec);
+        m->gexec = nullptr;
+      }
+    }
+    m->last_stage = 3;
+    m->flags_valid = false;
+    return DG_OK;
+  }
   if (m->st == nullptr) {  // the legacy default stream cannot be captured
     dg_status s = enqueue_step(m, indicator, tvb_M);
     m->last_stage = 3;

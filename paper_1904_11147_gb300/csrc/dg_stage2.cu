@@ -93,28 +93,6 @@ void pack(const dgt::Tabs& t, double* h) {
   for (int k = 0; k < 4; ++k) h[S::DX + k] = h[S::DY + k] = d[k];
 }
 
-// Doubled values at the Q Gauss points of sum_t e_t psi_t / psi_0 (KQ: sqrt(2) psi_t).
-template <int N>
-__device__ __forceinline__ void eval_gauss2(const double (&e)[N + 1], const double* __restrict__ kq, const Reg64& K,
-                                            double (&out)[N + 1]) {
-  constexpr int Q = N + 1;
-#pragma unroll
-  for (int q = 0; q < Q / 2; ++q) {
-    const double* c = kq + q * (N + 1);
-    double ev = e[0];
-    if constexpr (N >= 2) ev = fma(c[2], e[2], ev);
-    if constexpr (N == 3) {
-      const double od = fma(c[3], e[3], K.mul(c[1], e[1]));
-      out[q] = K.add(ev, od);
-      out[Q - 1 - q] = K.sub(ev, od);
-    } else {
-      out[q] = fma(c[1], e[1], ev);
-      out[Q - 1 - q] = fma(-c[1], e[1], ev);
-    }
-  }
-  if constexpr (N == 2) out[1] = fma(kq[(N + 1) + 2], e[2], e[0]);
-}
-
 // y sums relative to the outermost weight, psi_b (or psi_b') of even parity: over S = sums of
 // symmetric pairs (and the middle point), of odd parity: over D = differences
 template <int N>
@@ -125,11 +103,6 @@ __device__ __forceinline__ double rel_sum(bool even, const double (&S)[(N + 1) /
   else return even ? fma(kap, S[1], S[0]) : fma(kap, D[1], D[0]);
 }
 
-// what the kernels need of gamma
-struct Gamma {
-  double gm1, hgm1, sg;  // gamma - 1, -(gamma - 1) / 2, sqrt(gamma)
-};
-
 // Velocities, pressure and reciprocal density of a 2D Euler state (m1, m2: momentum).
 __device__ __forceinline__ void euler_state(double rho, double m1, double m2, double E, const double* __restrict__ c,
                                             int gm1, int hgm1, const Reg64& K, double& r, double& v1, double& v2,
@@ -138,27 +111,6 @@ __device__ __forceinline__ void euler_state(double rho, double m1, double m2, do
   v1 = K.mul(m1, r);
   v2 = K.mul(m2, r);
   p = fma(c[hgm1], fma(m1, v1, K.mul(m2, v2)), K.mul(c[gm1], E));  // (gamma-1)(E - rho |v|^2 / 2)
-}
-
-// sqrt(x) for the wave speed: the hardware's ~20-bit 1/sqrt(x) = y, t = x y = sqrt(x) (1-e)^(1/2)
-// with e = 1 - x y^2, and t (1 + e/2 + 3 e^2 / 8) (see sqrt_d; here without its final product).
-__device__ __forceinline__ double sqrt_t(double x, const Reg64& K, double c38, double half) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  if (b - 0x0010000000000000ull >= 0x7fe0000000000000ull) return sqrt(x);  // not a positive normal
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double t = K.mul(x, y), e = fma(-t, y, K.one);
-  return fma(t, K.mul(e, fma(c38, e, half)), t);
-}
-
-// larger of |a| and |b|, a NaN (a state without a real sound speed) if either is one: on the
-// bit patterns, where non-negative doubles order as integers and a NaN is largest (word by
-// word: a 64-bit mask would become an FP64 |x| instruction)
-__device__ __forceinline__ double max_speed(double a, double b) {
-  const unsigned ah = (unsigned)__double2hiint(a) & 0x7fffffffu, bh = (unsigned)__double2hiint(b) & 0x7fffffffu;
-  const unsigned al = (unsigned)__double2loint(a), bl = (unsigned)__double2loint(b);
-  const bool first = ah > bh || (ah == bh && al >= bl);
-  return __hiloint2double((int)(first ? ah : bh), (int)(first ? al : bl));
 }
 
 // Tiles: chunk Tile::x0 of kFaceChunk faces of the instance, row by row; Tile::pad = 0 for x

@@ -30,6 +30,54 @@ __device__ __forceinline__ double rcp_k(double x, const Reg64& K) {
   return fma(y, fma(e, e, e), y);
 }
 
+// what the kernels need of gamma
+struct Gamma {
+  double gm1, hgm1, sg;  // gamma - 1, -(gamma - 1) / 2, sqrt(gamma)
+};
+
+// sqrt(x) for the wave speed: the hardware's ~20-bit 1/sqrt(x) = y, t = x y = sqrt(x) (1-e)^(1/2)
+// with e = 1 - x y^2, and t (1 + e/2 + 3 e^2 / 8) (see sqrt_d; here without its final product).
+__device__ __forceinline__ double sqrt_t(double x, const Reg64& K, double c38, double half) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  if (b - 0x0010000000000000ull >= 0x7fe0000000000000ull) return sqrt(x);  // not a positive normal
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double t = K.mul(x, y), e = fma(-t, y, K.one);
+  return fma(t, K.mul(e, fma(c38, e, half)), t);
+}
+
+// larger of |a| and |b|, a NaN (a state without a real sound speed) if either is one: on the
+// bit patterns, where non-negative doubles order as integers and a NaN is largest (word by
+// word: a 64-bit mask would become an FP64 |x| instruction)
+__device__ __forceinline__ double max_speed(double a, double b) {
+  const unsigned ah = (unsigned)__double2hiint(a) & 0x7fffffffu, bh = (unsigned)__double2hiint(b) & 0x7fffffffu;
+  const unsigned al = (unsigned)__double2loint(a), bl = (unsigned)__double2loint(b);
+  const bool first = ah > bh || (ah == bh && al >= bl);
+  return __hiloint2double((int)(first ? ah : bh), (int)(first ? al : bl));
+}
+
+// Doubled values at the Q Gauss points of sum_t e_t psi_t / psi_0 (KQ: sqrt(2) psi_t).
+template <int N>
+__device__ __forceinline__ void eval_gauss2(const double (&e)[N + 1], const double* __restrict__ kq, const Reg64& K,
+                                            double (&out)[N + 1]) {
+  constexpr int Q = N + 1;
+#pragma unroll
+  for (int q = 0; q < Q / 2; ++q) {
+    const double* c = kq + q * (N + 1);
+    double ev = e[0];
+    if constexpr (N >= 2) ev = fma(c[2], e[2], ev);
+    if constexpr (N == 3) {
+      const double od = fma(c[3], e[3], K.mul(c[1], e[1]));
+      out[q] = K.add(ev, od);
+      out[Q - 1 - q] = K.sub(ev, od);
+    } else {
+      out[q] = fma(c[1], e[1], ev);
+      out[Q - 1 - q] = fma(-c[1], e[1], ev);
+    }
+  }
+  if constexpr (N == 2) out[1] = fma(kq[(N + 1) + 2], e[2], e[0]);
+}
+
 // Tables of one limiter (degree N, CSWENO or parent) as the kernels keep them in shared memory.
 template <int N>
 struct LimTab {
@@ -44,7 +92,8 @@ struct LimTab {
   static constexpr int CA = PG0 + 1;            // x part of the subcell averages times psi_0: [4] SA[last][n] psi_0
   static constexpr int CR = CA + 4;             // y part over psi_0: [4] SA[last][n] / psi_0
   static constexpr int P0 = CR + 4;             // psi_0
-  static constexpr int SIZE = (P0 + 2) / 2 * 2;
+  static constexpr int CS = P0 + 1;             // 1D subcell averages: [4] SA[last][n]
+  static constexpr int SIZE = (CS + 4 + 1) / 2 * 2;
 };
 
 // the largest of them, one row per degree
@@ -74,6 +123,7 @@ inline void pack_lim(const dgt::Tabs& t, double* h) {
     const double v = n <= N ? t.SA[2 * N][n] : 0.0;
     h[L::CA + n] = v * p0;
     h[L::CR + n] = v / p0;
+    h[L::CS + n] = v;
   }
   h[L::P0] = p0;
 }
