@@ -2,7 +2,8 @@
 //
 //   k_stage2    one stage of Eq. (5) fused in one kernel per tile (halo warps, shared
 //               faces), an autotuner alternative to the split stage (dg_stage2.cu)
-//   k_flag2     TVB minmod indicator + ballot/scan compaction of troubled cells
+//   k_flag2     TVB minmod indicator (FP32 screen, FP64 where that is undecided) + ballot/scan
+//               compaction of troubled cells
 //   k_project2  initial L2 projection (Eq. (2))
 //   k_speed2    largest characteristic speed over the cell means
 //
@@ -57,6 +58,7 @@ static_assert(Off<3>::END == Lay<1>::SIZE + Lay<2>::SIZE + Lay<3>::SIZE, "table 
 constexpr int kTabSize = Off<3>::END;
 
 __constant__ double c_tab[kTabSize];
+__constant__ float c_tef[3][10], c_tnf[3][10], c_c00f;  // TE, TN and C00 in FP32 (TVB screen)
 
 #define T(x) c_tab[(x)]
 
@@ -467,96 +469,226 @@ __global__ void __launch_bounds__((TYS + 3) * 32, 1)
 // formed without fused multiply-adds and in the order of a plain serial sum over the
 // modes, so the decision is reproducible bit for bit; products whose table factor is
 // exactly zero (psi_b(0) for odd b) are skipped, which leaves every partial sum unchanged.
+//
+// In FP64 that is 42 additions and products per variable (P2), bound by the FP64 pipe.  Nearly
+// every comparison is far from a tie, so an FP32 screen with error margins decides them first
+// (tvb_screen) and only cells with a comparison inside its margins take the FP64 pass.
 
+// The FP64 decision of one cell, variable and direction (0: x, 1: y): bit 0 troubled, bit 1
+// near threshold.
+template <int PDE, int N>
+__device__ __noinline__ int tvb_cell(const double* __restrict__ U, const Inst& I, int inst, int ix, int iy, int v,
+                                     int dir, long long ctot, int bc, double M, const double* __restrict__ bcd) {
+  using O = Off<N>;
+  constexpr int NP = np_of(2, N);
+  const double c00 = T(O::C00);
+  const double* P = U + (long long)(v * NP) * ctot;
+  const long long g = I.off + (long long)iy * I.nx + ix;
+  bool near = false;
+  // a neighbour's U_00: periodic wrap, outflow ghosts have the boundary cell's mean, kBcDmr
+  // ghosts follow dmr_ghost
+  auto nb_u00 = [&](int jx, int jy) -> double {
+    if (bc == 0) {
+      jx = jx < 0 ? jx + I.nx : (jx >= I.nx ? jx - I.nx : jx);
+      jy = jy < 0 ? jy + I.ny : (jy >= I.ny ? jy - I.ny : jy);
+    } else if (bc == kBcDmr && (jx < 0 || jx >= I.nx || jy < 0 || jy >= I.ny)) {
+      const Ghost gh = dmr_ghost(I, inst, jx, jy, bcd, dmr_time(bcd, inst, 0));
+      if (gh.c) return 2.0 * gh.c[v];
+      return neg_if(__ldg(P + I.off + (long long)gh.jy * I.nx + gh.jx), gh.fv && v == 2);
+    } else {
+      jx = jx < 0 ? 0 : (jx >= I.nx ? I.nx - 1 : jx);
+      jy = jy < 0 ? 0 : (jy >= I.ny ? I.ny - 1 : jy);
+    }
+    return __ldg(P + I.off + (long long)jy * I.nx + jx);
+  };
+  const double h = dir == 0 ? I.hx : I.hy;
+  const long long mh2 = __double_as_longlong(M * h * h);
+  const double mean = __dmul_rn(__ldg(P + g), c00);
+  const double mL = __dmul_rn(dir == 0 ? nb_u00(ix - 1, iy) : nb_u00(ix, iy - 1), c00);
+  const double mR = __dmul_rn(dir == 0 ? nb_u00(ix + 1, iy) : nb_u00(ix, iy + 1), c00);
+  // values at the midpoints of the two edges.  The serial sums start from their first term
+  // (0 + x = x up to the sign of a zero, which no decision below depends on).
+  double up = 0.0, um = 0.0;
+#pragma unroll
+  for (int m = 0; m < NP; ++m) {
+    const int n = dir == 0 ? mode_a(m) : mode_b(m), t = dir == 0 ? mode_b(m) : mode_a(m);
+    if (t & 1) continue;  // psi_t(0) = 0
+    // lower = (-1)^n upper, term by term
+    const double p = __dmul_rn(__ldg(P + (long long)m * ctot + g), dir == 0 ? T(O::TE + m) : T(O::TN + m));
+    up = m == 0 ? p : __dadd_rn(up, p);
+    um = m == 0 ? p : ((n & 1) ? __dsub_rn(um, p) : __dadd_rn(um, p));
+  }
+  const double dp = __dsub_rn(mR, mean), dm = __dsub_rn(mean, mL);
+  int fl = tvb_changes_bits(__dsub_rn(up, mean), dp, dm, mh2, near);
+  fl |= tvb_changes_bits(__dsub_rn(mean, um), dp, dm, mh2, near);
+  return fl | (near ? 2 : 0);
+}
+
+// ---- FP32 screen (exactness argument).  With m the mean, d a mean difference and
+// a = edge value - mean of the FP64 decision, S = sum_{n>=1} |U_n t_n| (t_n: table values):
+//   - a: the FP64 value is within (NP + 1) 2^-53 (|m| + S) < 2^-49 (|m| + S) of the exact
+//     sum_{n>=1} U_n t_n (U_0's product is the mean's, bit for bit).  In FP32 every U_n is
+//     truncated (2^-23) and every product and sum rounded (2^-24, at most 10 of them):
+//     within 2^-20 S.  Margin 2^-19 S + 2^-46 |m|.
+//   - d: a mean is kept as two floats, its leading 24 bits and the rest, exact to 2^-47 |m|;
+//     the differences of the parts and their sum round relative to the result (2^-24 each),
+//     the FP64 means and difference to 2^-52 |m|.  Margin 2^-21 |d| + 2^-44 max |m|.
+//   - every margin also holds 2^-100 for parts below the float range; infinities and NaN
+//     satisfy none of the comparisons below.
+// A test is decided when its comparisons hold with the margins and the windows of
+// tvb_changes_bits (2^-37 relative, 2^-39 of the largest magnitude) to spare: then the FP64
+// test decides the same and is not near a threshold.
+// double -> float by truncation without branches: values below 2^-126 give at most 2^-126,
+// those above the float range (and NaN) an infinity or a NaN.
+__device__ __forceinline__ float trunc_f(double x) {
+  const int hi = __double2hiint(x);
+  const int e = min(max((hi & 0x7fffffff) - (896 << 20), 0), 255 << 20);
+  return __uint_as_float(__funnelshift_l((unsigned)__double2loint(x), (unsigned)e, 3) | ((unsigned)hi & 0x80000000u));
+}
+struct Mean2 {  // U_00 (the mean over psi_0^2) as leading part and rest
+  float h, l;
+};
+__device__ __forceinline__ Mean2 split_mean(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const int e = (int)((hi >> 20) & 0x7ff) - 1023;
+  Mean2 r;
+  r.h = trunc_f(x);
+  // low 29 bits times 2^(e - 52), in range for |x| in [2^-60, 2^120]; outside the rest is made
+  // a NaN, which leaves the cell to FP64 (0 has none)
+  const float sc = __uint_as_float((unsigned)(e - 52 + 127) << 23);
+  const float l = __uint2float_rn(lo & 0x1fffffffu) * sc;
+  r.l = __uint_as_float(__float_as_uint(l) | (hi & 0x80000000u));
+  if (e < -60 || e > 120) r.l = (hi << 1) | lo ? __uint_as_float(0x7fc00000u) : 0.0f;
+  return r;
+}
+__device__ __forceinline__ float mean_diff(Mean2 a, Mean2 b) { return (a.h - b.h) + (a.l - b.l); }
+
+// The two tests of one direction (bit 0: the FP64 test finds a change; bit 1: undecided).
+// a0, a1, ma: edge values minus mean (mean minus edge value) and margin; dp, dm, md: the mean
+// differences and their margin; mlo, mhi: bounds of M h^2.
+__device__ __forceinline__ int tvb_screen(float a0, float a1, float ma, float dp, float dm, float md, float mlo,
+                                          float mhi) {
+  const float p = fabsf(dp), q = fabsf(dm), mp = fmaf(p, 0x1p-21f, md), mq = fmaf(q, 0x1p-21f, md);
+  const float plo = p - mp, qlo = q - mq, phi = p + mp, qhi = q + mq;
+  const float lo2 = fminf(plo, qlo), hi2 = fminf(phi, qhi), top2 = fmaxf(phi, qhi);
+  const bool same = (dp > 0.0f) == (dm > 0.0f);
+  int r = 0;
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const float a = k ? a1 : a0, fa = fabsf(a), lo = fa - ma, hi = fa + ma;
+    const float top = fmaxf(hi, top2) * 0x1p-38f;
+    const bool sure = lo > mhi && plo > top && qlo > top;  // above M h^2, no mean difference near zero
+    const bool agree = same && (a > 0.0f) == (dp > 0.0f);
+    const bool yes = sure && (!agree || lo > hi2 * (1.0f + 0x1p-20f));
+    const bool no = hi < mlo || (sure && agree && hi < lo2 * (1.0f - 0x1p-20f));
+    r |= yes ? 1 : (no ? 0 : 2);
+  }
+  return r;
+}
+
+// One thread per cell of a 32 x 8 tile: screen, then the block's undecided cells (listed in
+// shared memory, so that they fill whole warps) in FP64.  The tile's means and those of the
+// cells around it are split once, into shared memory.
+// Measured: 1024^2 Euler P2 0.07 ms (0.35 ms with every cell in FP64), P3 batch of 1.10 M
+// cells 0.09 ms (0.49).
 template <int PDE, int N>
 __global__ void __launch_bounds__(256)
     k_flag2(const double* __restrict__ U, const Inst* __restrict__ insts, const Tile* __restrict__ tiles,
             long long ctot, int bc, double M, unsigned char* __restrict__ flags, Counters* cnt,
             int* __restrict__ list_cell, int* __restrict__ list_inst, const double* __restrict__ bcd) {
-  using O = Off<N>;
-  constexpr int V = nv_of(2, PDE), NP = np_of(2, N);
+  constexpr int V = nv_of(2, PDE), NP = np_of(2, N), BX = TX + 2, BY = TY + 2;
   const Tile tile = tiles[blockIdx.x];
   const Inst I = insts[tile.inst];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int ix = tile.x0 + lane, iy = tile.y0 + w;
   const bool active = ix < I.nx && iy < I.ny;
-  const double c00 = T(O::C00);
-  int fl = 0;
-  bool near = false;
-  long long g = active ? I.off + (long long)iy * I.nx + ix : 0;
-  // every cell's means go to shared memory once; the neighbours inside the tile read them
-  // there, those outside it (and ghosts) form them from their U_00 as before
-  __shared__ double s_mean[V][TY][TX];
-  if (active) {
+  const long long g = active ? I.off + (long long)iy * I.nx + ix : 0;
+  __shared__ Mean2 s_mean[V][BY][BX];
+  __shared__ unsigned char s_todo[TX * TY];
+  __shared__ int s_res[TX * TY];
+  __shared__ int s_n;
+  __shared__ float s_mh2[2];  // M h^2, truncated
+  if (threadIdx.x == 0) {
+    s_n = 0;
+    s_mh2[0] = trunc_f(M * I.hx * I.hx);
+    s_mh2[1] = trunc_f(M * I.hy * I.hy);
+  }
+  for (int k = threadIdx.x; k < BX * BY; k += TX * TY) {
+    const int cy = k / BX, cx = k % BX;
+    int jx = tile.x0 + cx - 1, jy = tile.y0 + cy - 1;
+    if (jx > I.nx || jy > I.ny || ((cx == 0 || cx == BX - 1) && (cy == 0 || cy == BY - 1))) continue;
+    if (bc == 0) {
+      jx = jx < 0 ? jx + I.nx : (jx >= I.nx ? jx - I.nx : jx);
+      jy = jy < 0 ? jy + I.ny : (jy >= I.ny ? jy - I.ny : jy);
+    } else {  // outflow ghosts have the boundary cell's mean
+      jx = jx < 0 ? 0 : (jx >= I.nx ? I.nx - 1 : jx);
+      jy = jy < 0 ? 0 : (jy >= I.ny ? I.ny - 1 : jy);
+    }
+    const double* p = U + I.off + (long long)jy * I.nx + jx;
 #pragma unroll
-    for (int v = 0; v < V; ++v) s_mean[v][w][lane] = __dmul_rn(__ldg(U + (long long)(v * NP) * ctot + g), c00);
+    for (int v = 0; v < V; ++v) s_mean[v][cy][cx] = split_mean(__ldg(p + (long long)(v * NP) * ctot));
   }
   __syncthreads();
+  int fl = 0;
   if (active) {
-    // neighbour cells (outflow ghosts have the boundary cell's mean)
-    auto nb = [&](int jx, int jy) -> long long {
-      if (bc == 0) {
-        jx = jx < 0 ? jx + I.nx : (jx >= I.nx ? jx - I.nx : jx);
-        jy = jy < 0 ? jy + I.ny : (jy >= I.ny ? jy - I.ny : jy);
-      } else {
-        jx = jx < 0 ? 0 : (jx >= I.nx ? I.nx - 1 : jx);
-        jy = jy < 0 ? 0 : (jy >= I.ny ? I.ny - 1 : jy);
-      }
-      return I.off + (long long)jy * I.nx + jx;
-    };
-    const long long gW = nb(ix - 1, iy), gE = nb(ix + 1, iy), gS = nb(ix, iy - 1), gN = nb(ix, iy + 1);
-    const bool inW = lane > 0, inE = lane < TX - 1 && ix + 1 < I.nx;
-    const bool inS = w > 0, inN = w < TY - 1 && iy + 1 < I.ny;
-    // kBcDmr: the neighbours' U_00 (W, E, S, N) follow dmr_ghost where they lie outside
-    // (decided again per variable: only boundary cells of such meshes take this path)
-    const bool dmr = bc == kBcDmr && (ix == 0 || iy == 0 || ix == I.nx - 1 || iy == I.ny - 1);
-    auto nb_u00 = [&](int k, const double* P, long long gk, int v) -> double {
-      if (!dmr) return __ldg(P + gk);
-      const int jx = ix + (k == 0 ? -1 : (k == 1 ? 1 : 0)), jy = iy + (k == 2 ? -1 : (k == 3 ? 1 : 0));
-      if (jx >= 0 && jx < I.nx && jy >= 0 && jy < I.ny) return __ldg(P + gk);
-      const Ghost gh = dmr_ghost(I, tile.inst, jx, jy, bcd, dmr_time(bcd, tile.inst, 0));
-      if (gh.c) return 2.0 * gh.c[v];
-      return neg_if(__ldg(P + I.off + (long long)gh.jy * I.nx + gh.jx), gh.fv && v == 2);
-    };
-    const long long mx2 = __double_as_longlong(M * I.hx * I.hx), my2 = __double_as_longlong(M * I.hy * I.hy);
-#pragma unroll 1
-    for (int v = 0; v < V; ++v) {  // one variable at a time keeps the kernel at 4 blocks per SM
-      const double* P = U + (long long)(v * NP) * ctot;
-      const double mean = s_mean[v][w][lane];
-      const double mW = inW ? s_mean[v][w][lane - 1] : __dmul_rn(nb_u00(0, P, gW, v), c00);
-      const double mE = inE ? s_mean[v][w][lane + 1] : __dmul_rn(nb_u00(1, P, gE, v), c00);
-      const double mS = inS ? s_mean[v][w - 1][lane] : __dmul_rn(nb_u00(2, P, gS, v), c00);
-      const double mN = inN ? s_mean[v][w + 1][lane] : __dmul_rn(nb_u00(3, P, gN, v), c00);
-      // the serial sums start from their first term (0 + x = x up to the sign of a zero,
-      // which no decision below depends on)
-      double uE = 0.0, uW = 0.0, uN = 0.0, uS = 0.0;
-      bool firstE = true, firstN = true;
+    // the double Mach reflection's ghosts are left to FP64
+    if (bc == kBcDmr && (ix == 0 || iy == 0 || ix == I.nx - 1 || iy == I.ny - 1)) fl = 2;
+    const float xlo = s_mh2[0] * (1.0f - 0x1p-20f), xhi = fmaf(s_mh2[0], 1.0f + 0x1p-20f, 0x1p-100f);
+    const float ylo = s_mh2[1] * (1.0f - 0x1p-20f), yhi = fmaf(s_mh2[1], 1.0f + 0x1p-20f, 0x1p-100f);
 #pragma unroll
-      for (int m = 0; m < NP; ++m) {
+    for (int v = 0; v < V; ++v) {
+      const double* P = U + (long long)(v * NP) * ctot + g;
+      // edge values minus the mean: parts odd and even in the normal degree, and the sum of magnitudes
+      float ox = 0.0f, ex = 0.0f, oy = 0.0f, ey = 0.0f, sx = 0.0f, sy = 0.0f;
+#pragma unroll
+      for (int m = 1; m < NP; ++m) {
         const int a = mode_a(m), b = mode_b(m);
-        const double ck = __ldg(P + (long long)m * ctot + g);
-        if (!(b & 1)) {  // psi_b(0) != 0: east/west products (west = (-1)^a east)
-          const double pe = __dmul_rn(ck, T(O::TE + m));
-          uE = firstE ? pe : __dadd_rn(uE, pe);
-          uW = firstE ? ((a & 1) ? -pe : pe) : ((a & 1) ? __dsub_rn(uW, pe) : __dadd_rn(uW, pe));
-          firstE = false;
+        if ((a & 1) && (b & 1)) continue;  // psi_a(0) = psi_b(0) = 0
+        const float u = trunc_f(__ldg(P + (long long)m * ctot));
+        if (!(b & 1)) {
+          const float t = u * c_tef[N - 1][m];
+          if (a & 1) ox += t;
+          else ex += t;
+          sx += fabsf(t);
         }
-        if (!(a & 1)) {  // psi_a(0) != 0: north/south products (south = (-1)^b north)
-          const double pn = __dmul_rn(ck, T(O::TN + m));
-          uN = firstN ? pn : __dadd_rn(uN, pn);
-          uS = firstN ? ((b & 1) ? -pn : pn) : ((b & 1) ? __dsub_rn(uS, pn) : __dadd_rn(uS, pn));
-          firstN = false;
+        if (!(a & 1)) {
+          const float t = u * c_tnf[N - 1][m];
+          if (b & 1) oy += t;
+          else ey += t;
+          sy += fabsf(t);
         }
       }
-      const double dpx = __dsub_rn(mE, mean), dmx = __dsub_rn(mean, mW);
-      const double dpy = __dsub_rn(mN, mean), dmy = __dsub_rn(mean, mS);
-      fl |= tvb_changes_bits(__dsub_rn(uE, mean), dpx, dmx, mx2, near);
-      fl |= tvb_changes_bits(__dsub_rn(mean, uW), dpx, dmx, mx2, near);
-      fl |= tvb_changes_bits(__dsub_rn(uN, mean), dpy, dmy, my2, near);
-      fl |= tvb_changes_bits(__dsub_rn(mean, uS), dpy, dmy, my2, near);
+      const Mean2 mC = s_mean[v][w + 1][lane + 1], mW = s_mean[v][w + 1][lane], mE = s_mean[v][w + 1][lane + 2];
+      const Mean2 mS = s_mean[v][w][lane + 1], mN = s_mean[v][w + 2][lane + 1];
+      // in units of U_00 the mean is U_00 psi_0^2; the differences below take that factor
+      const float c = c_c00f, am = fabsf(mC.h) * c;
+      const float bx = fmaf(fmaxf(am, c * fmaxf(fabsf(mE.h), fabsf(mW.h))), 0x1p-44f, 0x1p-100f);
+      const float by = fmaf(fmaxf(am, c * fmaxf(fabsf(mN.h), fabsf(mS.h))), 0x1p-44f, 0x1p-100f);
+      const float rm = fmaf(am, 0x1p-46f, 0x1p-100f);
+      fl |= tvb_screen(ox + ex, ox - ex, fmaf(sx, 0x1p-19f, rm), c * mean_diff(mE, mC), c * mean_diff(mC, mW), bx, xlo, xhi);
+      fl |= tvb_screen(oy + ey, oy - ey, fmaf(sy, 0x1p-19f, rm), c * mean_diff(mN, mC), c * mean_diff(mC, mS), by, ylo, yhi);
     }
-    flags[g] = (unsigned char)(fl | (near ? 2 : 0));  // bit 0 troubled, bit 1 near threshold
+    if (fl & 2) {
+      s_todo[atomicAdd(&s_n, 1)] = (unsigned char)threadIdx.x;
+      s_res[threadIdx.x] = 0;
+    }
   }
+  __syncthreads();
+  // (a cell's variables and directions on neighbouring threads: the block waits for a few
+  // cells, so the chain of dependent FP64 operations is kept short)
+  for (int k = threadIdx.x; k < s_n * 2 * V; k += TX * TY) {
+    const int t = s_todo[k / (2 * V)], v = (k >> 1) % V, dir = k & 1;
+    const int r = tvb_cell<PDE, N>(U, I, tile.inst, tile.x0 + (t & 31), tile.y0 + (t >> 5), v, dir, ctot, bc, M, bcd);
+    if (r) atomicOr(&s_res[t], r);
+  }
+  __syncthreads();
+  bool near = false;
+  if (fl & 2) {
+    fl = s_res[threadIdx.x];
+    near = (fl & 2) != 0;
+  }
+  fl &= 1;
+  if (active) flags[g] = (unsigned char)(fl | (near ? 2 : 0));  // bit 0 troubled, bit 1 near threshold
   block_compact(fl, near ? 1 : 0, g, tile.inst, cnt, list_cell, list_inst);
 }
 
@@ -638,7 +770,19 @@ cudaError_t upload_tables2(const dgt::Tabs* tabs /* [3] for N = 1..3 */) {
   k2::pack<1>(tabs[0], h);
   k2::pack<2>(tabs[1], h);
   k2::pack<3>(tabs[2], h);
-  return cudaMemcpyToSymbol(k2::c_tab, h, sizeof(h));
+  static float te[3][10], tn[3][10];
+  for (int n = 0; n < 3; ++n)
+    for (int m = 0; m < np_of(2, n + 1); ++m) {
+      const int base = n == 0 ? k2::Off<1>::TE : (n == 1 ? k2::Off<2>::TE : k2::Off<3>::TE);
+      const int bn = n == 0 ? k2::Off<1>::TN : (n == 1 ? k2::Off<2>::TN : k2::Off<3>::TN);
+      te[n][m] = (float)h[base + m];
+      tn[n][m] = (float)h[bn + m];
+    }
+  const float c00 = (float)h[k2::Off<1>::C00];
+  cudaError_t e = cudaMemcpyToSymbol(k2::c_tab, h, sizeof(h));
+  if (e == cudaSuccess) e = cudaMemcpyToSymbol(k2::c_tef, te, sizeof(te));
+  if (e == cudaSuccess) e = cudaMemcpyToSymbol(k2::c_tnf, tn, sizeof(tn));
+  return e != cudaSuccess ? e : cudaMemcpyToSymbol(k2::c_c00f, &c00, sizeof(c00));
 }
 
 #define DG_DISPATCH2(PDE, N, CALL) \
