@@ -55,11 +55,9 @@ cudaError_t prepare_mlp(int dim, int pde, int N, int FP);
 void launch_features(int dim, int pde, int N, const LaunchArgs& a, double c0, float* X);
 void launch_label(int dim, int pde, int N, const LaunchArgs& a, double c0, const int* lc, const int* li,
                   const Counters* cnt, const double* lim, float* label, int nblocks);
-void launch_mlp_fb(cudaStream_t st, const float* X, const unsigned char* y, long long B, int F, const float* params,
-                   float pw, float* h1, float* d1, float* h2, float* d2, float* dz, float* loss);
 long long mlp_wgrad_chunks(long long B);
-void launch_mlp_wgrad(cudaStream_t st, const float* X, long long B, int F, const float* h1, const float* d1,
-                      const float* h2, const float* d2, const float* dz, float* part, float* grad);
+void launch_mlp_grad(cudaStream_t st, const float* X, const unsigned char* y, long long B, int F, const float* params,
+                     float pw, float* part, float* loss, float* grad);
 void launch_mlp_forward(cudaStream_t st, const float* X, long long B, int F, const float* params, float* z);
 void launch_mlp_adam(cudaStream_t st, float* params, const float* grad, float* m1, float* m2, int P, float lr, int t);
 void launch_mlp_export(cudaStream_t st, const float* params, int F, int FP, void* W1b, float* b1, void* W2b, float* b2,
@@ -1281,7 +1279,6 @@ struct dg_mlp {
   float *params = nullptr, *grad = nullptr, *m1 = nullptr, *m2 = nullptr, *loss = nullptr;
   void* infer = nullptr;  // BF16 W1 [32][FP], BF16 W2 [32][32], FP32 b1, b2, w3, b3
   long long cap = 0;
-  float *h1 = nullptr, *d1 = nullptr, *h2 = nullptr, *d2 = nullptr, *dz = nullptr;
   float* part = nullptr;  // per-chunk weight gradients [chunks][P]
 };
 
@@ -1321,7 +1318,7 @@ extern "C" size_t dg_mlp_param_count(const dg_mlp* n) { return n ? (size_t)n->P 
 extern "C" dg_status dg_mlp_destroy(dg_mlp* n) {
   if (!n) return DG_OK;
   cudaFree(n->params); cudaFree(n->grad); cudaFree(n->m1); cudaFree(n->m2); cudaFree(n->loss); cudaFree(n->infer);
-  cudaFree(n->h1); cudaFree(n->d1); cudaFree(n->h2); cudaFree(n->d2); cudaFree(n->dz); cudaFree(n->part);
+  cudaFree(n->part);
   delete n;
   return DG_OK;
 }
@@ -1396,13 +1393,9 @@ extern "C" dg_status dg_mlp_set_params(dg_mlp* n, const float* in, size_t count)
 
 static dg_status mlp_backward(dg_mlp* n, const float* X, const uint8_t* y, int64_t B, float pw) {
   if (B > n->cap) {
-    cudaFree(n->h1); cudaFree(n->d1); cudaFree(n->h2); cudaFree(n->d2); cudaFree(n->dz); cudaFree(n->part);
-    n->h1 = n->d1 = n->h2 = n->d2 = n->dz = n->part = nullptr;
-    const size_t hb = sizeof(float) * kHidden * (size_t)B;
-    if (cudaMalloc(&n->h1, hb) != cudaSuccess || cudaMalloc(&n->d1, hb) != cudaSuccess ||
-        cudaMalloc(&n->h2, hb) != cudaSuccess || cudaMalloc(&n->d2, hb) != cudaSuccess ||
-        cudaMalloc(&n->dz, sizeof(float) * (size_t)B) != cudaSuccess ||
-        cudaMalloc(&n->part, sizeof(float) * (size_t)n->P * (size_t)mlp_wgrad_chunks(B)) != cudaSuccess) {
+    cudaFree(n->part);
+    n->part = nullptr;
+    if (cudaMalloc(&n->part, sizeof(float) * (size_t)n->P * (size_t)mlp_wgrad_chunks(B)) != cudaSuccess) {
       cudaGetLastError();
       n->cap = 0;
       return fail(DG_ENOMEM, "training scratch for %lld samples", (long long)B);
@@ -1410,8 +1403,7 @@ static dg_status mlp_backward(dg_mlp* n, const float* X, const uint8_t* y, int64
     n->cap = B;
   }
   CK(cudaMemsetAsync(n->loss, 0, sizeof(float), n->st));
-  launch_mlp_fb(n->st, X, y, B, n->F, n->params, pw, n->h1, n->d1, n->h2, n->d2, n->dz, n->loss);
-  launch_mlp_wgrad(n->st, X, B, n->F, n->h1, n->d1, n->h2, n->d2, n->dz, n->part, n->grad);
+  launch_mlp_grad(n->st, X, y, B, n->F, n->params, pw, n->part, n->loss, n->grad);
   CK(cudaGetLastError());
   return DG_OK;
 }
