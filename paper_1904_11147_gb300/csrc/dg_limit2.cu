@@ -12,10 +12,15 @@
 // the result is added to, and the eigenvector products run on 2N differences instead of
 // 2N+1 averages.  Structural zeros of the subcell averages are used (a half of a cell has
 // no part of an even mode, a whole cell only that of psi_0), and the arithmetic has the
-// three-register form of dg_weno.cuh.  Per troubled cell the Euler kernel takes about 4,000
-// FP64 lane instructions for P2 and 8,900 for P3 (7,200 and 14,600 with averages, one
-// reciprocal per stencil and dense subcell sums); 6.9 and 15.8 ns per cell measured on 517k
-// P2 and 602k P3 cells (12.9 and 27.7 ns in that form), 95 % of the pipe's rate.
+// three-register form of dg_weno.cuh, whose reconstruction leaves only the smoothness
+// indicators and the final quotients to the FP64 pipe.
+//
+// Per troubled cell of a 512^2 Euler mesh (half its cells troubled): P2 5.6 ns, P3 14 ns.
+// With the reconstruction wholly in FP64: 7.4 and 16; on averages instead of differences,
+// with a reciprocal per stencil and dense subcell sums: 13 and 28.  The FP64 pipe is busy
+// 82 % (P2) and 69 % (P3) of the time, the rest is the latency of the integer chains at
+// 8 to 12 warps per SM; more warps with fewer registers (5, 6 or 8 blocks per SM) changed
+// nothing.
 #include "dg_shared.cuh"
 #include "dg_weno.cuh"
 

@@ -9,6 +9,9 @@
 // included -- and tables are read from shared memory into registers.
 #pragma once
 
+#include <cmath>
+#include <cstring>
+
 #include "dg_common.cuh"
 #include "tables.h"
 
@@ -84,8 +87,9 @@ struct LimTab {
   static constexpr int N1 = N + 1, NG = N == 1 ? 2 : 4;
   static constexpr int ONE = 0, NZ = 1;
   static constexpr int BF = 2;                  // [2][6] bform
-  static constexpr int WH = BF + 12;            // [NG][N1]
-  static constexpr int WC = WH + NG * N1;       // [NG][N1][N]
+  static constexpr int BR = BF + 12;            // brel as U64f (integers): significand, exponent
+  static constexpr int WH = BR + 2;             // [NG][N1] wh 2^63 (integers)
+  static constexpr int WC = WH + NG * N1;       // [NG][N1][N] wc 2^62 (signed integers)
   static constexpr int QS = WC + NG * N1 * N;   // [2] qsp
   static constexpr int PG = QS + 2;             // [NG][N1] w_g psi_n(r_g)
   static constexpr int PG0 = PG + NG * N1;      // sum_g w_g psi_0
@@ -107,13 +111,19 @@ inline void pack_lim(const dgt::Tabs& t, double* h) {
   h[L::NZ] = -0.0;
   for (int r = 0; r < 2; ++r)
     for (int k = 0; k < 6; ++k) h[L::BF + 6 * r + k] = t.bform[r][k];
+  auto put = [&](int k, unsigned long long v) { std::memcpy(h + k, &v, sizeof(v)); };
+  int be;
+  const double bf = std::frexp(t.brel, &be);  // in [1/2, 1): significand 2^64 bf, brel = m 2^(be - 64)
+  put(L::BR, (unsigned long long)std::ldexp(bf, 64));
+  put(L::BR + 1, (unsigned long long)(long long)be);
   h[L::QS] = t.qsp[0];
   h[L::QS + 1] = t.qsp[1];
   h[L::PG0] = 0.0;
   for (int g = 0; g < L::NG; ++g) {
     for (int i = 0; i <= N; ++i) {
-      h[L::WH + g * L::N1 + i] = t.wh[g][i];
-      for (int j = 0; j < N; ++j) h[L::WC + (g * L::N1 + i) * N + j] = t.wc[g][i][j];
+      put(L::WH + g * L::N1 + i, (unsigned long long)std::ldexp(t.wh[g][i], 63));
+      for (int j = 0; j < N; ++j)
+        put(L::WC + (g * L::N1 + i) * N + j, (unsigned long long)(long long)std::llrint(std::ldexp(t.wc[g][i][j], 62)));
       h[L::PG + g * L::N1 + i] = t.rw[g] * t.psiG[g][i];
     }
     h[L::PG0] += t.rw[g] * t.psiG[g][0];
@@ -128,23 +138,64 @@ inline void pack_lim(const dgt::Tabs& t, double* h) {
   h[L::P0] = p0;
 }
 
+// ----------------------------------------------------------------------------- reconstruction
+// Integer arithmetic of the reconstruction.  In the time of one FP64 instruction (67 clocks
+// per warp and SM sub-partition) the integer pipes do a 64-bit product and more, so everything
+// behind the smoothness indicators runs there, on positive floating-point numbers m 2^e with a
+// 64-bit significand (products and weights: 11 bits more than a double) and on fixed-point sums.
+struct U64f {
+  unsigned long long m;  // in [2^63, 2^64), or 0
+  int e;
+};
+__device__ __forceinline__ U64f unpack_pos(double x) {  // of a positive normal number; e is biased
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  return U64f{((unsigned long long)(__funnelshift_l(lo, hi, 11) | 0x80000000u) << 32) | (lo << 11), (int)(hi >> 20)};
+}
+// a b / 2^64; relative error below 2^-62
+__device__ __forceinline__ U64f mul_n(U64f a, U64f b) {
+  const unsigned long long m = __umul64hi(a.m, b.m);
+  const int up = (long long)m >= 0;  // in [2^62, 2^63)
+  return U64f{m << up, a.e + b.e - up};
+}
+// t 2^q as a double (rounded to nearest, ties away); out of range: 0 or infinity
+__device__ __forceinline__ double pack_s64(long long t, int q) {
+  const unsigned long long a = t < 0 ? 0ull - (unsigned long long)t : (unsigned long long)t;
+  const int z = __clzll((long long)a), e = 1086 - z + q;
+  const unsigned long long m = a << (z & 63);
+  unsigned long long bits = ((unsigned long long)(unsigned)(e - 1) << 52) + (m >> 11) + ((m >> 10) & 1ull);
+  if (e < 1 || a == 0) bits = 0ull;
+  if (e > 2046 && a != 0) bits = 0x7ff0000000000000ull;
+  return __longlong_as_double((long long)(bits | ((unsigned long long)t & 0x8000000000000000ull)));
+}
+
 // Steps 2-5: u_g - avg[N] at the Step 1 points from the 2N differences d (see Tabs::bform,
-// wc, wh).  Per call 20 / 71 / 142 FP64 instructions for N = 1, 2, 3.
+// wc, wh).
 //
-// The weights need 1 / D_i^2-like ratios only up to a common factor, so instead of a
-// reciprocal per stencil P_i is the product of the other stencils' D.  That overflows for
-// extreme data, so where any D reaches 2^150 (or is not a number) the reciprocals are
-// taken, scaled by the power of two that brings the largest into [1, 2).
+//   b_i   (eps + beta_i) / M_i, a sum of squares, in FP64
+//   P_i   the weights' 1 / (eps + beta_i)^2 up to a common factor: the product of the other
+//         stencils' squares, as U64f (any magnitude of the data)
+//   X_ij  P_i d_{i+j}, sign apart
+//   T_g, S_g   sum wc X and sum wh P in 64-bit fixed point: all X are shifted to the largest
+//         one's exponent (below 2^62, so a sum of |wc| / 4 < 1/4 each stays below 2^63), all P
+//         to theirs.  A term loses at most 2^-62 of the largest one, and every product at most
+//         one unit of the sum, half of it on average (added back at the start).
+//   u_g - avg[N] = T_g / S_g, in FP64
+// FP64 instructions per call: 10 / 27 / 64 for N = 1, 2, 3 (20 / 71 / 142 with all of it in
+// FP64), next to some 150 / 700 / 1,500 integer ones.  Limiter of 130k P2 cells 974 -> 730 us,
+// of 140k P3 cells 2,200 -> 1,950 us, Burgers P2 224 -> 139 us.
+//
 // SPLIT: the CSWENO P3 rule with one negative weight at each inner point.  With T and S the
-// sums of wc P d and wh P over the positive (+) and the negative (-) weights, the difference
-// of the two normalised parts of the split is
+// sums over the positive (+) and the negative (-) weights, the difference of the two
+// normalised parts of the split is
 //   [T+ (den1 + q0 S-) - T- (q1 S+ - den2)] / (den1 den2), den1 = 2 S+ + S-, den2 = S+ + 2 S-.
 template <int N, bool SPLIT>
 __device__ __forceinline__ void weno_diff(const double (&d)[2 * N], const double* __restrict__ tab, const Reg64& K,
                                           double (&out)[N == 1 ? 2 : 4]) {
   using L = LimTab<N>;
   constexpr int N1 = N + 1, NG = L::NG;
-  double D[N1];
+  const unsigned long long* itab = reinterpret_cast<const unsigned long long*>(tab);
+  bool bad = false;  // a difference that is not finite
+  U64f D[N1];
 #pragma unroll
   for (int i = 0; i < N1; ++i) {
     const bool mir = 2 * i > N;
@@ -161,93 +212,98 @@ __device__ __forceinline__ void weno_diff(const double (&d)[2 * N], const double
       const double v = fma(f[3], e1, fma(f[4], e2, e0)), w = fma(f[5], e2, e1);
       b = fma(v, v, fma(K.mul(f[2], w), w, fma(f[1], K.mul(e2, e2), f[0])));
     }
-    D[i] = K.mul(b, b);
+    bad = bad || ((unsigned)__double2hiint(b) & 0x7fffffffu) > 0x7ff00000u;
+    D[i] = unpack_pos(b);
+    // the outer stencils' M over the inner ones'
+    if (N > 1 && (i == 0 || i == N)) D[i] = mul_n(D[i], U64f{itab[L::BR], (int)itab[L::BR + 1]});
+    D[i] = mul_n(D[i], D[i]);
   }
-  int hi = __double2hiint(D[0]);
-#pragma unroll
-  for (int i = 1; i < N1; ++i) hi = max(hi, __double2hiint(D[i]));
-  double P[N1];
-  if (hi < (1023 + 150) << 20) {  // D >= eps^2 / M^2 > 0, so the bit patterns order as integers
-    if constexpr (N == 1) {
-      P[0] = D[1];
-      P[1] = D[0];
-    } else if constexpr (N == 2) {
-      P[0] = K.mul(D[1], D[2]);
-      P[1] = K.mul(D[0], D[2]);
-      P[2] = K.mul(D[0], D[1]);
-    } else {
-      const double a = K.mul(D[0], D[1]), b = K.mul(D[2], D[3]);
-      P[0] = K.mul(D[1], b);
-      P[1] = K.mul(D[0], b);
-      P[2] = K.mul(D[3], a);
-      P[3] = K.mul(D[2], a);
-    }
+  U64f P[N1];
+  if constexpr (N == 1) {
+    P[0] = D[1];
+    P[1] = D[0];
+  } else if constexpr (N == 2) {
+    P[0] = mul_n(D[1], D[2]);
+    P[1] = mul_n(D[0], D[2]);
+    P[2] = mul_n(D[0], D[1]);
   } else {
-    int top = 0;
-#pragma unroll
-    for (int i = 0; i < N1; ++i) {
-      P[i] = 1.0 / D[i];
-      top = max(top, __double2hiint(P[i]) & 0x7fffffff);
-    }
-    top = (top >> 20) < 2047 ? (top >> 20) : 1023;
-    const double s = __hiloint2double((2046 - top) << 20, 0);  // 2^(1023 - top)
-#pragma unroll
-    for (int i = 0; i < N1; ++i) P[i] *= s;
+    const U64f a = mul_n(D[0], D[1]), b = mul_n(D[2], D[3]);
+    P[0] = mul_n(D[1], b);
+    P[1] = mul_n(D[0], b);
+    P[2] = mul_n(D[3], a);
+    P[3] = mul_n(D[2], a);
   }
-  double X[N1][N];
+  U64f dm[2 * N];
+  unsigned neg = 0;  // bit k: d_k < 0
 #pragma unroll
-  for (int i = 0; i < N1; ++i)
+  for (int k = 0; k < 2 * N; ++k) {
+    const unsigned hi = (unsigned)__double2hiint(d[k]), ab = hi & 0x7fffffffu;
+    bad = bad || ab >= 0x7ff00000u;
+    neg |= (hi >> 31) << k;
+    dm[k] = unpack_pos(__hiloint2double((int)ab, __double2loint(d[k])));
+    if (ab < 0x00100000u) dm[k] = U64f{0ull, -(1 << 20)};  // zero (or subnormal)
+  }
+  U64f X[N1][N];
+  int ex = -(1 << 20), ep = P[0].e;
 #pragma unroll
-    for (int j = 0; j < N; ++j) X[i][j] = K.mul(P[i], d[i + j]);
+  for (int i = 0; i < N1; ++i) {
+    ep = max(ep, P[i].e);
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      X[i][j] = mul_n(P[i], dm[i + j]);
+      if (dm[i + j].m != 0ull) ex = max(ex, X[i][j].e);
+    }
+  }
+  long long Xf[N1][N];
+  unsigned long long Pf[N1];
+#pragma unroll
+  for (int i = 0; i < N1; ++i) {
+    Pf[i] = P[i].m >> min(ep - P[i].e + 2, 63);
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      const long long x = (long long)(X[i][j].m >> min(max(ex - X[i][j].e + 2, 0), 63));
+      Xf[i][j] = (neg >> (i + j)) & 1u ? -x : x;
+    }
+  }
+  // T_g 2^64 = sum Xf (wc 2^62), S_g 2^64 = sum Pf (wh 2^63); X = Xf 2^(ex + 2 + 64 - 1086) and
+  // P = Pf 2^(ep + 2) up to P's common factor: u_g - avg[N] = T_g / S_g 2^(ex - ep - 1021)
+  const int q = min(max(ex - ep - 1021, -8000), 8000);
   double num[NG], den[NG];
 #pragma unroll
   for (int g = 0; g < NG; ++g) {
-    constexpr int kNone = -1;
-    const int neg = SPLIT ? dgt::weno_neg(N, g, false) : kNone;
-    const int ref = dgt::weno_ref(N, g);
-    const double* wc = tab + L::WC + g * N1 * N;
-    const double* wh = tab + L::WH + g * N1;
-    double T = 0.0, S = P[ref];
-    bool first = true;
+    const int ng = SPLIT ? dgt::weno_neg(N, g, false) : -1, ref = dgt::weno_ref(N, g);
+    const long long* wc = reinterpret_cast<const long long*>(itab) + L::WC + g * N1 * N;
+    const unsigned long long* wh = itab + L::WH + g * N1;
+    long long Tp = ng < 0 ? N1 * N / 2 : N * N / 2, Tm = N / 2;
+    unsigned long long Sp = Pf[ref] >> 1, Sm = 0;
 #pragma unroll
     for (int i = 0; i < N1; ++i) {
-      if (i == neg) continue;
-      if (i != ref) S = fma(wh[i], P[i], S);
+      if (i == ng) Sm = __umul64hi(wh[i], Pf[i]);
+      else if (i != ref) Sp += __umul64hi(wh[i], Pf[i]);
 #pragma unroll
       for (int j = 0; j < N; ++j) {
-        T = first ? K.mul(wc[i * N + j], X[i][j]) : fma(wc[i * N + j], X[i][j], T);
-        first = false;
+        const long long t = __mul64hi(wc[i * N + j], Xf[i][j]);
+        if (i == ng) Tm += t;
+        else Tp += t;
       }
     }
-    if (neg < 0) {
-      num[g] = T;
-      den[g] = S;
+    if (ng < 0) {
+      num[g] = pack_s64(Tp, q);
+      den[g] = pack_s64((long long)Sp, 0);
     } else {
-      const double Sm = K.mul(wh[neg], P[neg]);
-      double Tm = K.mul(wc[neg * N], X[neg][0]);
-#pragma unroll
-      for (int j = 1; j < N; ++j) Tm = fma(wc[neg * N + j], X[neg][j], Tm);
-      const double den1 = K.add(S, K.add(S, Sm)), den2 = K.add(Sm, K.add(S, Sm));
-      num[g] = fma(T, fma(tab[L::QS], Sm, den1), -K.mul(Tm, fma(tab[L::QS + 1], S, -den2)));
+      const double T = pack_s64(Tp, q), Tn = pack_s64(Tm, q), S = pack_s64((long long)Sp, 0), Sn = pack_s64((long long)Sm, 0);
+      const double den1 = K.add(S, K.add(S, Sn)), den2 = K.add(Sn, K.add(S, Sn));
+      num[g] = fma(T, fma(tab[L::QS], Sn, den1), -K.mul(Tn, fma(tab[L::QS + 1], S, -den2)));
       den[g] = K.mul(den1, den2);
     }
   }
-  // one range check for all points (see rcp_d)
-  bool ok = true;
 #pragma unroll
-  for (int g = 0; g < NG; ++g)
-    ok = ok && ((unsigned)__double2hiint(den[g]) & 0x7fffffffu) - 0x00100000u < 0x7fc00000u;
-  if (ok) {
-#pragma unroll
-    for (int g = 0; g < NG; ++g) {
-      double y;
-      asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(den[g]));
-      const double e = fma(-den[g], y, K.one);
-      out[g] = K.mul(num[g], fma(y, fma(e, e, e), y));
-    }
-  } else {
-#pragma unroll
-    for (int g = 0; g < NG; ++g) out[g] = num[g] / den[g];
+  for (int g = 0; g < NG; ++g) {  // S_g lies in [2^50, 2^63): no range check (see rcp_d)
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(den[g]));
+    const double e = fma(-den[g], y, K.one);
+    out[g] = K.mul(num[g], fma(y, fma(e, e, e), y));
+    if (bad) out[g] = __longlong_as_double(0x7ff8000000000000LL);
   }
 }
 

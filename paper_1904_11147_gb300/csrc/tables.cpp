@@ -307,15 +307,16 @@ int build_tables(int N, Tabs* t, bool parent) {
         for (int c = 0; c < 6; ++c) t->bform[i][c] = (double)f[c];
     }
   }
-  for (int g = 0; g < t->NG; ++g) {
-    const int r = weno_ref(N, g);
-    const ld ref = Gm[g][r] / (Mb[r] * Mb[r]);
+  t->brel = N == 1 ? 1.0 : (double)(Mb[0] / Mb[1]);
+  for (int g = 0; g < t->NG; ++g)
     for (int i = 0; i <= N; ++i) {
-      const ld h = fabsl(Gm[g][i]) / (Mb[i] * Mb[i]) / ref;
+      const ld h = fabsl(Gm[g][i]) / Gm[g][weno_ref(N, g)];
       t->wh[g][i] = (double)h;
       for (int j = 0; j < N; ++j) t->wc[g][i][j] = (double)(h * Eg[g][i][j]);
+      if (t->wh[g][i] >= 2.0) return 3;  // the ranges of the kernels' fixed-point sums
+      for (int j = 0; j < N; ++j)
+        if (std::fabs(t->wc[g][i][j]) >= 2.0) return 3;
     }
-  }
   // subcell averages (Fig. 1): N equal parts of each neighbour, troubled cell whole
   {
     ld qx[kMaxQ], qw[kMaxQ];

@@ -43,16 +43,16 @@ struct Tabs {
   // for i <= N/2 and mirrored for the others, beta_i / M is a sum of squares,
   //   N = 1: e_0^2;  N = 2: (e_0 + k e_1)^2 + o e_1^2;
   //   N = 3: (e_0 + k e_1 + l e_2)^2 + m (e_1 + n e_2)^2 + o e_2^2,
-  // with the same constants for stencils i and N - i (class min(i, N - i)); the factors M go
-  // into the weights.  bform = {eps / M, o, m, k, l, n}.
+  // with the same constants for stencils i and N - i (class min(i, N - i)).  bform = {eps / M, o, m, k, l, n}.
   double bform[2][6];
-  // p_i(x_g) - avg[N] = sum_j E_gij d_{i+j}.  With P_i proportional to the reciprocal of
-  // (eps / M + beta_i / M)^2: wh[g][i] = gamma_gi / M_i^2 over its value at the reference
-  // stencil weno_ref(N, g) and wc[g][i][j] = wh[g][i] E_gij, so that
+  // p_i(x_g) - avg[N] = sum_j E_gij d_{i+j}.  With P_i proportional to 1 / (eps + beta_i)^2 and
+  // wh[g][i] = gamma_gi over its value at the reference stencil weno_ref(N, g),
+  // wc[g][i][j] = wh[g][i] E_gij,
   //   u_g - avg[N] = sum_ij wc_gij P_i d_{i+j} / sum_i wh_gi P_i.
   // At a point with one negative weight (sigma+ and sigma- of the split) wh and wc of that
   // stencil are taken with |gamma|; qsp = {4 sigma+ - sigma- - 1, 4 sigma- - sigma+ + 1}.
-  double wh[kMaxG][kMaxN + 1], wc[kMaxG][kMaxN + 1][kMaxN], qsp[2];
+  // brel = M of the outer stencils over M of the inner ones (1 for N = 1).
+  double wh[kMaxG][kMaxN + 1], wc[kMaxG][kMaxN + 1][kMaxN], qsp[2], brel;
   // initial projection: (N+4)-point Gauss rule
   int QP;
   double px[kMaxQ], pw[kMaxQ], ppsi[kMaxQ][kMaxN + 1];
