@@ -7,9 +7,9 @@
 //            the stage combination.
 // Every face flux is computed once; all lanes of every warp do the same work.
 //
-// Bound: the FP64 pipe.  Point values are formed over psi_0 = 1/sqrt(2) and doubled
-// (2 sum_t (e_t / psi_0) psi_t(s) psi_0 = e_0 + sum_{t>=1} e_t sqrt(2) psi_t(s)), so the constant
-// term needs no multiplication; the fluxes are homogeneous in the state (Euler of degree 1,
+// Bound: the FP64 pipe.  Traces and volume point values are linear in the modes: they are
+// formed in fixed point on the integer pipes (dg_weno.cuh), over psi_0 = 1/sqrt(2) and doubled
+// (2 sum_t (e_t / psi_0) psi_t(s) psi_0 = e_0 + sum_{t>=1} e_t sqrt(2) psi_t(s)); the fluxes are homogeneous in the state (Euler of degree 1,
 // Burgers of degree 2), so the factor is taken back in the final scalings.  The Gauss points
 // are symmetric and psi_t has the parity of t: sums and differences over pairs of points.
 // Every quadrature sum is kept relative to its outermost weight (one product less), and all
@@ -17,11 +17,13 @@
 // block.  The density's volume term needs no quadrature: its flux is the momentum, a
 // polynomial.  Arithmetic in the three-register form of dg_weno.cuh.
 //
-// Measured per launch (Euler; with plain sums and products, constant operands, products
-// with every weight and 32-wide face tiles in parentheses): 1024^2 P2 face pass 0.87 ms
-// (1.09), cell pass 0.88 ms (1.19); P3 batch of 1.10 M cells 1.46 ms (1.84) and 1.98 ms
-// (3.18); 1537 x 1021 P1 0.80 ms (1.02) and 0.44 ms (0.66); FP64 pipe 88-95 % busy.
+// Measured per launch (Euler; in parentheses with the traces and point values in FP64, and
+// before that with plain sums and products, constant operands, products with every weight and
+// 32-wide face tiles): 1024^2 P2 face pass 0.70 ms (0.87, 1.09), cell pass 0.81 ms (0.88,
+// 1.19); P3 batch of 1.10 M cells 1.04 ms (1.46, 1.84) and 1.98 ms (1.98, 3.18); 1537 x 1021 P1
+// 0.68 ms (0.80, 1.02) and 0.44 ms (0.44, 0.66).
 #include <cmath>
+#include <cstring>
 
 #include "dg_shared.cuh"
 #include "dg_weno.cuh"
@@ -36,9 +38,10 @@ struct STab {
   static constexpr int ONE = 0, NZ = 1, C38 = 2, HALF = 3;
   static constexpr int GM1 = 4, HGM1 = 5, SG = 6;   // gamma - 1, -(gamma - 1) / 2, sqrt(gamma) (set by the block)
   static constexpr int RA = 7, RB = 8;              // weights of u^n and of the stage's input (set by the block)
-  static constexpr int KP1 = 9;                     // [N1] sqrt(2) psi_n(1)
-  static constexpr int KQ = KP1 + N1;               // [NX][N1] sqrt(2) psi_n(x_q), x_q <= 0
-  static constexpr int KAP = KQ + NX * N1;          // [N1] w psi_b at the second point over the first
+  static constexpr int KP1 = 9;                     // [N1] sqrt(2) psi_n(1) 2^61 (integers)
+  static constexpr int KQ = KP1 + N1;               // [NX][N1] sqrt(2) psi_n(x_q) 2^62, x_q <= 0 (integers)
+  static constexpr int KD = KQ + NX * N1;           // [NX][N1] sqrt(2) psi_n(x_q) in FP64
+  static constexpr int KAP = KD + NX * N1;          // [N1] w psi_b at the second point over the first
   static constexpr int KAD = KAP + N1;              // [N1] w psi_b' at the second point over the first
   // times (2/hx) dt times the stage's weight times 2^-d
   static constexpr int XF = KAD + N1;
@@ -66,11 +69,18 @@ void pack(const dgt::Tabs& t, double* h) {
   h[S::NZ] = -0.0;
   h[S::C38] = 0.375;
   h[S::HALF] = 0.5;
+  auto put = [&](int k, double v) {
+    const long long i = std::llrint(v);
+    std::memcpy(h + k, &i, sizeof(i));
+  };
   auto wp = [&](int q, int b) { return t.gw[q] * t.psi_q[q][b]; };
   auto wd = [&](int q, int b) { return t.gw[q] * t.dpsi_q[q][b]; };
   for (int n = 0; n < N1; ++n) {
-    h[S::KP1 + n] = t.kp1[n];
-    for (int q = 0; q < NX; ++q) h[S::KQ + q * N1 + n] = t.kq[q][n];
+    put(S::KP1 + n, std::ldexp(t.kp1[n], 61));
+    for (int q = 0; q < NX; ++q) {
+      put(S::KQ + q * N1 + n, std::ldexp(t.kq[q][n], 62));
+      h[S::KD + q * N1 + n] = t.kq[q][n];
+    }
     h[S::KAP + n] = wp(1, n) / wp(0, n);
     h[S::KAD + n] = n ? wd(1, n) / wd(0, n) : 0.0;
   }
@@ -117,7 +127,7 @@ __device__ __forceinline__ void euler_state(double rho, double m1, double m2, do
 // faces (k = 0..nx, j < ny), 1 for y faces (k < nx, j = 0..ny).  Face k of a row lies between
 // cells k-1 and k.  (Chunks of the face index instead of 32-wide tiles: a row of nx + 1 faces
 // left most lanes of its last warp idle, 6 % of all warps at nx = 512.)
-// FP64 instructions per face (Euler): 128, 222, 354 for P1, P2, P3.
+// FP64 instructions per face (Euler): 104, 166, 226 for P1, P2, P3.
 template <int PDE, int N>
 __global__ void __launch_bounds__(kFaceChunk) k_face2(const double* __restrict__ us, const Inst* __restrict__ insts,
                                                const Tile* __restrict__ tiles, long long ctot, int bc, Gamma gm,
@@ -143,6 +153,7 @@ __global__ void __launch_bounds__(kFaceChunk) k_face2(const double* __restrict__
   __syncthreads();
   if (j >= I.ny + dir) return;
   const Reg64 K{tab[T::ONE], tab[T::NZ]};
+  const long long* itab = reinterpret_cast<const long long*>(tab);
   // variables in the order (rho, normal momentum, tangential momentum, E) and modes by
   // (normal degree n, transverse degree t): the planes are read in that order
   double tr[2][Q][V];
@@ -189,17 +200,20 @@ __global__ void __launch_bounds__(kFaceChunk) k_face2(const double* __restrict__
         if (cst) x = m == 0 ? 2.0 * cst[pv] : 0.0;  // constant state: U_00 = 2 mean, no other mode
         u[m] = neg_if(x, ((fn && (n & 1)) != (ft && (t & 1))) != wall);
       }
-      double e[N1], val[Q];
+      // sums over the normal degree (an eighth; sum |KP1| < 8), then at the points (a quarter)
+      long long X[NP], e[N1], val[Q];
+      const int E = align_modes<NP>(u, X);
 #pragma unroll
       for (int t = 0; t <= N; ++t) {
-        double s = u[mode_idx(0, t)];
+        long long z = X[mode_idx(0, t)] >> 3;
 #pragma unroll
-        for (int n = 1; n <= N - t; ++n) s = fma(tab[T::KP1 + n], u[mode_idx(n, t)], s);
-        e[t] = s;
+        for (int n = 1; n <= N - t; ++n) z += __mul64hi(itab[T::KP1 + n], X[mode_idx(n, t)]);
+        e[t] = z;
       }
-      eval_gauss2<N>(e, tab + T::KQ, K, val);
+      eval_fix<N>(e, itab + T::KQ, val);
 #pragma unroll
-      for (int q = 0; q < Q; ++q) tr[side][q][v] = val[q];
+      for (int q = 0; q < Q; ++q)
+        tr[side][q][v] = E < 2047 ? pack_s64(val[q], E - 1079) : __longlong_as_double(0x7ff8000000000000LL);
     }
   }
   double G[Q][V];
@@ -242,10 +256,14 @@ __global__ void __launch_bounds__(kFaceChunk) k_face2(const double* __restrict__
   }
 }
 
-// One thread per cell; Tile::x0: chunk of kCellChunk cells of the instance.  FP64
-// instructions per cell (Euler, stages 2 and 3): 184, 473, 1060 for P1, P2, P3.
-// Two blocks per SM (at most 128 registers) except for Euler P3, which needs more registers
-// and keeps the cell's modes in shared memory (one slot per thread and mode).
+// One thread per cell; Tile::x0: chunk of kCellChunk cells of the instance.
+// Two blocks per SM (at most 128 registers) except for Euler P3; Euler P2 and P3 keep the cell's
+// modes in shared memory (one slot per thread and mode).  Point values in fixed point pay for
+// P2 (Euler 878 -> 809 us at 1024^2, Burgers 211 -> 198 us); P1 has too little to move (439 -> 470 us)
+// and P3 no registers for it (1.98 -> 2.74 ms): those stay in FP64.
+__host__ __device__ constexpr bool fixed_values(int N) { return N == 2; }
+__host__ __device__ constexpr bool smem_modes(int pde, int N) { return pde == 1 && N >= 2; }
+
 template <int PDE, int N>
 __global__ void __launch_bounds__(kCellChunk, (PDE == 1 && N == 3) ? 1 : 2)
     k_cell2(const double* __restrict__ un, const double* __restrict__ us, double* __restrict__ out,
@@ -276,20 +294,34 @@ __global__ void __launch_bounds__(kCellChunk, (PDE == 1 && N == 3) ? 1 : 2)
   if (iy >= I.ny) return;
   const Reg64 K{tab[T::ONE], tab[T::NZ]};
   const long long g = I.off + loc;
-  constexpr bool kSmemU = PDE == 1 && N == 3;
-  extern __shared__ double s_u[];
-  double ur[kSmemU ? 1 : V][kSmemU ? 1 : NP];
+  constexpr bool kFix = fixed_values(N), kSmemU = smem_modes(PDE, N);
+  const long long* itab = reinterpret_cast<const long long*>(tab);
+  extern __shared__ long long s_x[];  // the modes as doubles or aligned integers
+  long long xr[kSmemU ? 1 : V][kSmemU ? 1 : NP];
+  int E[V];
 #pragma unroll
-  for (int v = 0; v < V; ++v)
+  for (int v = 0; v < V; ++v) {
+    double u[NP];
+    long long X[NP];
 #pragma unroll
     for (int m = 0; m < NP; ++m) {
-      const double x = __ldg(us + (long long)(v * NP + m) * ctot + g);
-      if constexpr (kSmemU) s_u[(v * NP + m) * kCellChunk + threadIdx.x] = x;
-      else ur[v][m] = x;
+      u[m] = __ldg(us + (long long)(v * NP + m) * ctot + g);
+      X[m] = __double_as_longlong(u[m]);
     }
+    if constexpr (kFix) E[v] = align_modes<NP>(u, X);
+#pragma unroll
+    for (int m = 0; m < NP; ++m) {
+      if constexpr (kSmemU) s_x[(v * NP + m) * kCellChunk + threadIdx.x] = X[m];
+      else xr[v][m] = X[m];
+    }
+  }
+  auto x = [&](int v, int m) -> long long {
+    if constexpr (kSmemU) return s_x[(v * NP + m) * kCellChunk + threadIdx.x];
+    else return xr[v][m];
+  };
   auto u = [&](int v, int m) -> double {
-    if constexpr (kSmemU) return s_u[(v * NP + m) * kCellChunk + threadIdx.x];
-    else return ur[v][m];
+    if constexpr (kFix) return __ldg(us + (long long)(v * NP + m) * ctot + g);
+    else return __longlong_as_double(x(v, m));
   };
   // acc[v][m]: the stage's weight times dt times the right-hand side
   double acc[V][NP];
@@ -305,33 +337,56 @@ __global__ void __launch_bounds__(kCellChunk, (PDE == 1 && N == 3) ? 1 : 2)
 #pragma unroll
   for (int p = 0; p < NX; ++p) {
     const bool mid = (Q & 1) && p == Q / 2;
-    double tb[2][V][N1];  // over psi_0, at -x_p and x_p (parts even and odd in a)
+    double tb[kFix ? 1 : 2][kFix ? 1 : V][N1];  // FP64: over psi_0, at -x_p and x_p (parts even and odd in a)
+    if constexpr (!kFix) {
 #pragma unroll
-    for (int v = 0; v < V; ++v)
+      for (int v = 0; v < V; ++v)
 #pragma unroll
-      for (int b = 0; b <= N; ++b) {
-        const double* c = tab + T::KQ + p * N1;
-        double ev = u(v, mode_idx(0, b));
-        if (N - b >= 2) ev = fma(c[2], u(v, mode_idx(N - b >= 2 ? 2 : 0, b)), ev);
-        tb[0][v][b] = tb[1][v][b] = ev;
-        if (mid || b == N) continue;
-        const double u1 = u(v, mode_idx(b < N ? 1 : 0, b));
-        if (N - b >= 3) {
-          const double od = fma(c[3 <= N ? 3 : 0], u(v, mode_idx(N - b >= 3 ? 3 : 0, b)), K.mul(c[1], u1));
-          tb[0][v][b] = K.add(ev, od);
-          tb[1][v][b] = K.sub(ev, od);
-        } else {
-          tb[0][v][b] = fma(c[1], u1, ev);
-          tb[1][v][b] = fma(-c[1], u1, ev);
+        for (int b = 0; b <= N; ++b) {
+          const double* c = tab + T::KD + p * N1;
+          double ev = u(v, mode_idx(0, b));
+          if (N - b >= 2) ev = fma(c[N >= 2 ? 2 : 0], u(v, mode_idx(N - b >= 2 ? 2 : 0, b)), ev);
+          tb[0][v][b] = tb[1][v][b] = ev;
+          if (mid || b == N) continue;
+          const double u1 = u(v, mode_idx(b < N ? 1 : 0, b));
+          if (N - b >= 3) {
+            const double od = fma(c[3 <= N ? 3 : 0], u(v, mode_idx(N - b >= 3 ? 3 : 0, b)), K.mul(c[1], u1));
+            tb[0][v][b] = K.add(ev, od);
+            tb[1][v][b] = K.sub(ev, od);
+          } else {
+            tb[0][v][b] = fma(c[1], u1, ev);
+            tb[1][v][b] = fma(-c[1], u1, ev);
+          }
         }
-      }
+    }
     double Gs[V][N], Hs[V][N];  // of the column at -x_p
 #pragma unroll
     for (int side = 0; side < 2; ++side) {
       if (mid && side) break;
       double col[V][Q];
 #pragma unroll
-      for (int v = 0; v < V; ++v) eval_gauss2<N>(tb[side][v], tab + T::KQ, K, col[v]);
+      for (int v = 0; v < V; ++v) {
+        if constexpr (kFix) {
+          // x sums over psi_0 at -x_p (side 0) or x_p, a quarter (formed again for each side: the
+          // integer pipes have the time, the registers are short), then the y points
+          const long long* c = itab + T::KQ + p * N1;
+          long long tb[N1], val[Q];
+  #pragma unroll
+          for (int b = 0; b <= N; ++b) {
+            long long ev = x(v, mode_idx(0, b)) >> 2, od = 0;
+            if (N - b >= 2) ev += __mul64hi(c[N >= 2 ? 2 : 0], x(v, mode_idx(N - b >= 2 ? 2 : 0, b)));
+            if (!mid && b < N) od = __mul64hi(c[1], x(v, mode_idx(b < N ? 1 : 0, b)));
+            if (N - b >= 3) od += __mul64hi(c[3 <= N ? 3 : 0], x(v, mode_idx(N - b >= 3 ? 3 : 0, b)));
+            tb[b] = side == 0 ? ev + od : ev - od;
+          }
+          eval_fix<N>(tb, itab + T::KQ, val);
+  #pragma unroll
+          for (int q = 0; q < Q; ++q)
+            col[v][q] = E[v] < 2047 ? pack_s64(val[q], E[v] - 1080) : __longlong_as_double(0x7ff8000000000000LL);
+        } else {
+          eval_gauss2<N>(tb[side][v], tab + T::KD, K, col[v]);
+        }
+      }
       double F[V][Q], H[V][Q];
 #pragma unroll
       for (int q = 0; q < Q; ++q) {
@@ -437,8 +492,10 @@ __global__ void __launch_bounds__(kCellChunk, (PDE == 1 && N == 3) ? 1 : 2)
   }
 }
 
-// dynamic shared memory of the cell pass: the modes of its 256 cells for Euler P3
-constexpr size_t cell_smem(int pde, int N) { return pde == 1 && N == 3 ? sizeof(double) * 4 * 10 * kCellChunk : 0; }
+// dynamic shared memory of the cell pass: the modes of its 256 cells
+constexpr size_t cell_smem(int pde, int N) {
+  return smem_modes(pde, N) ? sizeof(long long) * 4 * ((N + 1) * (N + 2) / 2) * kCellChunk : 0;
+}
 
 template <int PDE, int N>
 void launch(const LaunchArgs& a, int stage, double dt_all, const Tile* face_tiles, int nface_tiles, double* fx,
@@ -463,8 +520,9 @@ cudaError_t upload_tables_stage2(const dgt::Tabs* tabs) {
 // opt in to more than 48 KB of dynamic shared memory (set per device, outside captures)
 cudaError_t prepare_stage2_split(int pde, int N) {
   if (!st2::cell_smem(pde, N)) return cudaSuccess;
-  return cudaFuncSetAttribute(st2::k_cell2<1, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)st2::cell_smem(pde, N));
+  const int bytes = (int)st2::cell_smem(pde, N);
+  return N == 2 ? cudaFuncSetAttribute(st2::k_cell2<1, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)
+                : cudaFuncSetAttribute(st2::k_cell2<1, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 
 int face_chunk2() { return st2::kFaceChunk; }

@@ -59,6 +59,61 @@ __device__ __forceinline__ double max_speed(double a, double b) {
   return __hiloint2double((int)(first ? ah : bh), (int)(first ? al : bl));
 }
 
+// ----------------------------------------------------------------------------- fixed point
+// Sums of modes times constants in 64-bit fixed point.  In the time of one FP64 instruction (67
+// clocks per warp and SM sub-partition) the integer pipes do several 64-bit products, and
+// they are idle otherwise.  The modes of a variable are aligned to the largest one (below
+// 2^62), so a sum's error is a few 2^-59 of the largest mode, where FP64 rounds each partial sum
+// to 2^-53 of itself.
+
+// t 2^q as a double (rounded to nearest, ties away); out of range: 0 or infinity
+__device__ __forceinline__ double pack_s64(long long t, int q) {
+  const unsigned long long a = t < 0 ? 0ull - (unsigned long long)t : (unsigned long long)t;
+  const int z = __clzll((long long)a), e = 1086 - z + q;
+  const unsigned long long m = a << (z & 63);
+  unsigned long long bits = ((unsigned long long)(unsigned)(e - 1) << 52) + (m >> 11) + ((m >> 10) & 1ull);
+  if (e < 1 || a == 0) bits = 0ull;
+  if (e > 2046 && a != 0) bits = 0x7ff0000000000000ull;
+  return __longlong_as_double((long long)(bits | ((unsigned long long)t & 0x8000000000000000ull)));
+}
+
+// X[m] 2^(E - 1084) = u[m], |X| < 2^62; values 2^-62 below the largest are dropped, and so are
+// numbers below 2^-958.  E >= 2047: a mode is not finite.
+template <int M>
+__device__ __forceinline__ int align_modes(const double (&u)[M], long long (&X)[M]) {
+  unsigned top = 64u << 20;
+#pragma unroll
+  for (int m = 0; m < M; ++m) top = max(top, (unsigned)__double2hiint(u[m]) & 0x7fffffffu);
+  const int E = (int)(top >> 20);
+#pragma unroll
+  for (int m = 0; m < M; ++m) {
+    const unsigned hi = (unsigned)__double2hiint(u[m]), lo = (unsigned)__double2loint(u[m]);
+    const unsigned long long w = ((unsigned long long)__funnelshift_l(lo, (hi & 0xfffffu) | 0x100000u, 9) << 32) | (lo << 9);
+    const long long x = (long long)(w >> min(E - (int)((hi >> 20) & 0x7ffu), 63)), s = (long long)((int)hi >> 31);
+    X[m] = (x ^ s) - s;
+  }
+  return E;
+}
+
+// A quarter of sum_t e_t KQ_qt at the Q Gauss points (KQ_q0 = 1); kq: KQ 2^62, rows of the
+// points <= 0.
+template <int N>
+__device__ __forceinline__ void eval_fix(const long long (&e)[N + 1], const long long* __restrict__ kq,
+                                         long long (&out)[N + 1]) {
+  constexpr int Q = N + 1;
+  const long long e0 = e[0] >> 2;
+#pragma unroll
+  for (int q = 0; q < Q / 2; ++q) {
+    const long long* c = kq + q * (N + 1);
+    long long ev = e0, od = __mul64hi(c[1], e[1]);
+    if constexpr (N >= 2) ev += __mul64hi(c[2], e[2]);
+    if constexpr (N == 3) od += __mul64hi(c[3], e[3]);
+    out[q] = ev + od;
+    out[Q - 1 - q] = ev - od;
+  }
+  if constexpr (N == 2) out[1] = e0 + __mul64hi(kq[(N + 1) + 2], e[2]);
+}
+
 // Doubled values at the Q Gauss points of sum_t e_t psi_t / psi_0 (KQ: sqrt(2) psi_t).
 template <int N>
 __device__ __forceinline__ void eval_gauss2(const double (&e)[N + 1], const double* __restrict__ kq, const Reg64& K,
@@ -157,17 +212,6 @@ __device__ __forceinline__ U64f mul_n(U64f a, U64f b) {
   const int up = (long long)m >= 0;  // in [2^62, 2^63)
   return U64f{m << up, a.e + b.e - up};
 }
-// t 2^q as a double (rounded to nearest, ties away); out of range: 0 or infinity
-__device__ __forceinline__ double pack_s64(long long t, int q) {
-  const unsigned long long a = t < 0 ? 0ull - (unsigned long long)t : (unsigned long long)t;
-  const int z = __clzll((long long)a), e = 1086 - z + q;
-  const unsigned long long m = a << (z & 63);
-  unsigned long long bits = ((unsigned long long)(unsigned)(e - 1) << 52) + (m >> 11) + ((m >> 10) & 1ull);
-  if (e < 1 || a == 0) bits = 0ull;
-  if (e > 2046 && a != 0) bits = 0x7ff0000000000000ull;
-  return __longlong_as_double((long long)(bits | ((unsigned long long)t & 0x8000000000000000ull)));
-}
-
 // Steps 2-5: u_g - avg[N] at the Step 1 points from the 2N differences d (see Tabs::bform,
 // wc, wh).
 //
