@@ -15,12 +15,10 @@
 // three-register form of dg_weno.cuh, whose reconstruction leaves only the smoothness
 // indicators and the final quotients to the FP64 pipe.
 //
-// Per troubled cell of a 512^2 Euler mesh (half its cells troubled): P2 5.6 ns, P3 14 ns.
-// With the reconstruction wholly in FP64: 7.4 and 16; on averages instead of differences,
-// with a reciprocal per stencil and dense subcell sums: 13 and 28.  The FP64 pipe is busy
-// 82 % (P2) and 69 % (P3) of the time, the rest is the latency of the integer chains at
-// 8 to 12 warps per SM; more warps with fewer registers (5, 6 or 8 blocks per SM) changed
-// nothing.
+// Per troubled cell of a 512^2 Euler mesh (half its cells troubled): P2 5.1 ns, P3 11 ns.
+// With the line reconstruction inlined in both sweeps: 5.6 and 14; with it wholly in FP64
+// besides: 7.4 and 16; on averages instead of differences, with a reciprocal per stencil and
+// dense subcell sums: 13 and 28.  The FP64 pipe is busy 89 % (P2) and 85 % (P3) of the time.
 #include "dg_shared.cuh"
 #include "dg_weno.cuh"
 
@@ -227,6 +225,22 @@ __device__ __forceinline__ void from_char(const Eig& e, double vn, double vt, co
   E = fma(e.H, s, fma(vn, t, fma(e.hq2, w[1], K.mul(vt, w[2]))));
 }
 
+// The reconstruction of one line: 2N differences p[k stride] in shared memory, replaced by the
+// values at the Step 1 points.  One copy for both sweeps: it is most of the kernel's code, and
+// inlined twice it ran out of the instruction cache (1024^2 P2 step 13.3 -> 12.5 ms, P3 batch of
+// 8 x 128 x 512 cells 37.5 -> 33.1 ms per step).  One lane per cell (Burgers) gains nothing from it.
+template <int N, bool SPLIT>
+__device__ __noinline__ void weno_line(double* p, int stride, const double* __restrict__ tab) {
+  using L = LimTab<N>;
+  const Reg64 K{tab[L::ONE], tab[L::NZ]};
+  double d[2 * N], r[L::NG];
+#pragma unroll
+  for (int k = 0; k < 2 * N; ++k) d[k] = p[k * stride];
+  weno_diff<N, SPLIT>(d, tab, K, r);
+#pragma unroll
+  for (int k = 0; k < L::NG; ++k) p[k * stride] = r[k];
+}
+
 // CSWENO or parent limiter for 2D Euler, four lanes per troubled cell: the list is often
 // short (a few cells per SM sub-partition), and a cell's work has four-way parallelism at
 // each step.  Lane q of a quad owns
@@ -244,9 +258,12 @@ __device__ __forceinline__ void from_char(const Eig& e, double vn, double vt, co
 // With a work counter (lq, zero at launch) a warp takes its next 8 cells from it, so the
 // work spreads over the resident warps whatever the grid.
 constexpr int kQuadThreads = 64;
+// Blocks per SM.  P3: 6 (168 registers) 31.9 ms per step of the batch above, 5 33.1, 8 32.5; P2: 8
+// (128 registers) 12.2 ms per 1024^2 step, 6 12.4.  P1 needs fewer registers than either allows.
+__host__ __device__ constexpr int quad_blocks(int N) { return N == 3 ? 6 : 8; }
 
 template <int N, bool PARENT>
-__global__ void __launch_bounds__(kQuadThreads)
+__global__ void __launch_bounds__(kQuadThreads, quad_blocks(N))
     k_limit2_euler(const double* __restrict__ U, const Inst* __restrict__ insts, long long ctot, int bc,
                    const int* __restrict__ list_cell, const int* __restrict__ list_inst,
                    const Counters* __restrict__ cnt, double* __restrict__ lim, long long cap, double gam,
@@ -321,20 +338,13 @@ __global__ void __launch_bounds__(kQuadThreads)
     __syncwarp();
     // x sweep: field q of every row; point values replace the differences
 #pragma unroll 1
-    for (int ky = 0; ky < NS; ++ky) {
-      double d[2 * N], r[NG];
-#pragma unroll
-      for (int k = 0; k < 2 * N; ++k) d[k] = S[ky * ROW + 4 * k + q];
-      weno_diff<N, SPLIT>(d, tab, K, r);
-#pragma unroll
-      for (int k = 0; k < NG; ++k) S[ky * ROW + 4 * k + q] = r[k];
-    }
+    for (int ky = 0; ky < NS; ++ky) weno_line<N, SPLIT>(S + ky * ROW + q, 4, tab);
     __syncwarp();
     double mid[4];  // the middle row's averages at x point q
     if (q < NG) {
       // back to conserved variables at x point q; y differences to characteristic fields
       double prev[4] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll
+#pragma unroll 1
       for (int ky = 0; ky < NS; ++ky) {
         double w[4], u[4];
 #pragma unroll
@@ -359,10 +369,10 @@ __global__ void __launch_bounds__(kQuadThreads)
       // y sweep of the column, projected in y: t_b = sum_g w_g psi_b(y_g) (u(y_g) - mid)
 #pragma unroll 1
       for (int f = 0; f < 4; ++f) {
-        double d[2 * N], r[NG];
+        double r[NG];
+        weno_line<N, SPLIT>(S + 4 * q + f, ROW, tab);
 #pragma unroll
-        for (int k = 0; k < 2 * N; ++k) d[k] = S[k * ROW + 4 * q + f];
-        weno_diff<N, SPLIT>(d, tab, K, r);
+        for (int k = 0; k < NG; ++k) r[k] = S[k * ROW + 4 * q + f];
         double sp[NG / 2], sm[NG / 2];  // the points are symmetric, psi_b has the parity of b
 #pragma unroll
         for (int k = 0; k < NG / 2; ++k) {
@@ -380,7 +390,7 @@ __global__ void __launch_bounds__(kQuadThreads)
           S[b * ROW + 4 * q + f] = t;
         }
       }
-#pragma unroll
+#pragma unroll 1
       for (int b = 0; b <= N; ++b) {
         double w[4], u[4];
 #pragma unroll

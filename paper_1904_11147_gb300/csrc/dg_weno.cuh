@@ -225,7 +225,7 @@ __device__ __forceinline__ U64f mul_n(U64f a, U64f b) {
 //         one unit of the sum, half of it on average (added back at the start).
 //   u_g - avg[N] = T_g / S_g, in FP64
 // FP64 instructions per call: 10 / 27 / 64 for N = 1, 2, 3 (20 / 71 / 142 with all of it in
-// FP64), next to some 150 / 700 / 1,500 integer ones.  Limiter of 130k P2 cells 974 -> 730 us,
+// FP64), next to some 150 / 700 / 1,500 integer ones.  With it, limiter of 130k P2 cells 974 -> 730 us,
 // of 140k P3 cells 2,200 -> 1,950 us, Burgers P2 224 -> 139 us.
 //
 // SPLIT: the CSWENO P3 rule with one negative weight at each inner point.  With T and S the
