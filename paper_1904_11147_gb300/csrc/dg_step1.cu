@@ -284,7 +284,7 @@ __device__ __forceinline__ void field1(const double (&d)[2 * N], const double* _
   using L = LimTab<N>;
   constexpr int NG = L::NG, N1 = N + 1;
   double r[NG];
-  weno_diff<N, N == 3>(d, lt, K, r);
+  weno_diff<N, N == 3, false>(d, lt, K, r);
 #pragma unroll
   for (int b = 1; b <= N; ++b) {
     double s = 0.0;
@@ -472,8 +472,8 @@ __global__ void __launch_bounds__(128)
 // a stage are listed in shared memory and their work spread over the block by (cell,
 // variable), (cell, difference) and (cell, field), so that a few troubled cells do not leave
 // most of the block's warps idle.
-// Measured per step, with five kernels per stage in parentheses: 160 Burgers P2 cells 22 us
-// (80), 64 x 800 Euler P3 cells 198 us (468).  Three blocks per SM (448 tiles of the latter on
+// Measured per step, with five kernels per stage in parentheses: 160 Burgers P2 cells 21 us
+// (80), 64 x 800 Euler P3 cells 180 us (468).  Three blocks per SM (448 tiles of the latter on
 // 152 SMs) bound the registers to 168; tiles of 84 cells would need a second wave.
 constexpr int kStepThreads = 128, kHalo = 6, kStepTile = kStepThreads - 2 * kHalo;
 

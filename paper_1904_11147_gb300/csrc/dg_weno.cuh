@@ -145,8 +145,9 @@ struct LimTab {
   static constexpr int BR = BF + 12;            // brel as U64f (integers): significand, exponent
   static constexpr int WH = BR + 2;             // [NG][N1] wh 2^63 (integers)
   static constexpr int WC = WH + NG * N1;       // [NG][N1][N] wc 2^62 (signed integers)
-  static constexpr int QS = WC + NG * N1 * N;   // [2] qsp
-  static constexpr int PG = QS + 2;             // [NG][N1] w_g psi_n(r_g)
+  static constexpr int QS = WC + NG * N1 * N;   // [2] qsp 2^59 (integers; qsp is 12.2 and 9.3)
+  static constexpr int QD = QS + 2;             // [2] qsp in FP64
+  static constexpr int PG = QD + 2;             // [NG][N1] w_g psi_n(r_g)
   static constexpr int PG0 = PG + NG * N1;      // sum_g w_g psi_0
   static constexpr int CA = PG0 + 1;            // x part of the subcell averages times psi_0: [4] SA[last][n] psi_0
   static constexpr int CR = CA + 4;             // y part over psi_0: [4] SA[last][n] / psi_0
@@ -171,8 +172,8 @@ inline void pack_lim(const dgt::Tabs& t, double* h) {
   const double bf = std::frexp(t.brel, &be);  // in [1/2, 1): significand 2^64 bf, brel = m 2^(be - 64)
   put(L::BR, (unsigned long long)std::ldexp(bf, 64));
   put(L::BR + 1, (unsigned long long)(long long)be);
-  h[L::QS] = t.qsp[0];
-  h[L::QS + 1] = t.qsp[1];
+  for (int r = 0; r < 2; ++r) h[L::QD + r] = t.qsp[r];
+  for (int r = 0; r < 2; ++r) put(L::QS + r, (unsigned long long)(long long)std::llrint(std::ldexp(t.qsp[r], 59)));
   h[L::PG0] = 0.0;
   for (int g = 0; g < L::NG; ++g) {
     for (int i = 0; i <= N; ++i) {
@@ -212,6 +213,31 @@ __device__ __forceinline__ U64f mul_n(U64f a, U64f b) {
   const int up = (long long)m >= 0;  // in [2^62, 2^63)
   return U64f{m << up, a.e + b.e - up};
 }
+// t / s 2^q as a double; the quotient before its rounding is within 2^-60 (relative).  1/s from
+// FP32's reciprocal Y (23 bits) and one third-order step, Y (1 + e + e^2) with e = 1 - s Y.
+__device__ __forceinline__ double quot_s64(long long t, unsigned long long s, int q) {
+  unsigned long long a = t < 0 ? 0ull - (unsigned long long)t : (unsigned long long)t;
+  const int zt = __clzll((long long)a), zs = __clzll((long long)s);
+  a <<= zt & 63;
+  s <<= zs & 63;
+  const unsigned hi = (unsigned)(s >> 32), lo = (unsigned)s;
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(__uint_as_float(0x3f800000u | ((hi >> 8) & 0x7fffffu))));
+  const unsigned yb = __float_as_uint(y), Y = yb >= 0x3f800000u ? 0xffffffffu : (yb << 8) | 0x80000000u;  // 2^95 / s
+  // e 2^63, rounded down: the reciprocal does not pass 2^64
+  const long long e = (long long)(0x7fffffffffffffffull - ((unsigned long long)hi * Y + __umulhi(lo, Y)));
+  const int eh = (int)(e >> 11);
+  const long long g = e + (((long long)eh * eh) >> 41);
+  const long long d = (((long long)(int)(g >> 12) * (long long)Y) >> 19) + (long long)__umulhi(((unsigned)g & 0xfffu) << 1, Y);
+  const unsigned long long h = __umul64hi(a, ((unsigned long long)Y << 32) + (unsigned long long)d);  // >= 2^62
+  const int up = (long long)h >= 0, b = 1023 + q - zt + zs - up;
+  const unsigned long long m = h << up;
+  unsigned long long bits = ((unsigned long long)(unsigned)(b - 1) << 52) + (m >> 11) + ((m >> 10) & 1ull);
+  if (b < 1 || t == 0) bits = 0ull;
+  if (b > 2046 && t != 0) bits = 0x7ff0000000000000ull;
+  return __longlong_as_double((long long)(bits | ((unsigned long long)t & 0x8000000000000000ull)));
+}
+
 // Steps 2-5: u_g - avg[N] at the Step 1 points from the 2N differences d (see Tabs::bform,
 // wc, wh).
 //
@@ -223,16 +249,23 @@ __device__ __forceinline__ U64f mul_n(U64f a, U64f b) {
 //         one's exponent (below 2^62, so a sum of |wc| / 4 < 1/4 each stays below 2^63), all P
 //         to theirs.  A term loses at most 2^-62 of the largest one, and every product at most
 //         one unit of the sum, half of it on average (added back at the start).
-//   u_g - avg[N] = T_g / S_g, in FP64
-// FP64 instructions per call: 10 / 27 / 64 for N = 1, 2, 3 (20 / 71 / 142 with all of it in
-// FP64), next to some 150 / 700 / 1,500 integer ones.  With it, limiter of 130k P2 cells 974 -> 730 us,
-// of 140k P3 cells 2,200 -> 1,950 us, Burgers P2 224 -> 139 us.
+//   u_g - avg[N] = T_g / S_g, in integers rounded once, or in FP64
+// FP64 instructions per call: 2 / 12 / 32 for N = 1, 2, 3 (10 / 27 / 64 with the quotient in
+// FP64, 20 / 71 / 142 with all of it), next to some 250 / 800 / 1,700 integer ones.  From all of it
+// in FP64 to FP64 quotients: limiter of 130k P2 cells 974 -> 730 us, of 140k P3 cells 2,200 ->
+// 1,950 us.  Integer quotients besides: 1024^2 P2 step 12.3 -> 11.1 ms, P3 batch of 8 x 128 x
+// 512 cells 31.8 -> 30.0 ms.
+//
+// INTQ: the quotient in integers (2D).  1D keeps it in FP64: its steps gain little (64 x 800 P3
+// cells 180 -> 171 us, 160 Burgers cells nothing), and long P3 shock-tube runs without
+// the positivity scaling depend on the last bit (of six FP64 runs of one of them, perturbed by
+// 1e-16 to 5e-16 each step, one lost positivity).
 //
 // SPLIT: the CSWENO P3 rule with one negative weight at each inner point.  With T and S the
 // sums over the positive (+) and the negative (-) weights, the difference of the two
 // normalised parts of the split is
 //   [T+ (den1 + q0 S-) - T- (q1 S+ - den2)] / (den1 den2), den1 = 2 S+ + S-, den2 = S+ + 2 S-.
-template <int N, bool SPLIT>
+template <int N, bool SPLIT, bool INTQ = true>
 __device__ __forceinline__ void weno_diff(const double (&d)[2 * N], const double* __restrict__ tab, const Reg64& K,
                                           double (&out)[N == 1 ? 2 : 4]) {
   using L = LimTab<N>;
@@ -312,7 +345,6 @@ __device__ __forceinline__ void weno_diff(const double (&d)[2 * N], const double
   // T_g 2^64 = sum Xf (wc 2^62), S_g 2^64 = sum Pf (wh 2^63); X = Xf 2^(ex + 2 + 64 - 1086) and
   // P = Pf 2^(ep + 2) up to P's common factor: u_g - avg[N] = T_g / S_g 2^(ex - ep - 1021)
   const int q = min(max(ex - ep - 1021, -8000), 8000);
-  double num[NG], den[NG];
 #pragma unroll
   for (int g = 0; g < NG; ++g) {
     const int ng = SPLIT ? dgt::weno_neg(N, g, false) : -1, ref = dgt::weno_ref(N, g);
@@ -331,22 +363,36 @@ __device__ __forceinline__ void weno_diff(const double (&d)[2 * N], const double
         else Tp += t;
       }
     }
-    if (ng < 0) {
-      num[g] = pack_s64(Tp, q);
-      den[g] = pack_s64((long long)Sp, 0);
+    if constexpr (!INTQ) {
+      double num, den;
+      if (ng < 0) {
+        num = pack_s64(Tp, q);
+        den = pack_s64((long long)Sp, 0);
+      } else {
+        const double T = pack_s64(Tp, q), Tn = pack_s64(Tm, q), S = pack_s64((long long)Sp, 0), Sn = pack_s64((long long)Sm, 0);
+        const double den1 = K.add(S, K.add(S, Sn)), den2 = K.add(Sn, K.add(S, Sn));
+        num = fma(T, fma(tab[L::QD], Sn, den1), -K.mul(Tn, fma(tab[L::QD + 1], S, -den2)));
+        den = K.mul(den1, den2);
+      }
+      double y;  // S_g lies in [2^50, 2^63): no range check (see rcp_d)
+      asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(den));
+      const double e = fma(-den, y, K.one);
+      out[g] = K.mul(num, fma(y, fma(e, e, e), y));
+    } else if (ng < 0) {
+      out[g] = quot_s64(Tp, Sp, q);
     } else {
-      const double T = pack_s64(Tp, q), Tn = pack_s64(Tm, q), S = pack_s64((long long)Sp, 0), Sn = pack_s64((long long)Sm, 0);
-      const double den1 = K.add(S, K.add(S, Sn)), den2 = K.add(Sn, K.add(S, Sn));
-      num[g] = fma(T, fma(tab[L::QS], Sn, den1), -K.mul(Tn, fma(tab[L::QS + 1], S, -den2)));
-      den[g] = K.mul(den1, den2);
+      // S+ and S- below 2^59 (the larger one from 2^58 on), T+ and T- below 2^63: a factor of T is
+      // below (2 + 1 + 12.3) 2^59 < 2^63
+      const long long* qs = reinterpret_cast<const long long*>(itab) + L::QS;
+      const int c = __clzll((long long)(Sp | Sm));
+      const long long A = (long long)((Sp << (c & 63)) >> 5), B = (long long)((Sm << (c & 63)) >> 5);
+      const long long den1 = A + A + B, den2 = A + B + B;
+      const long long ta = Tp ^ (Tp >> 63), tb = Tm ^ (Tm >> 63);
+      const int z = (__clzll(ta | tb) - 1) & 63;
+      const long long num = __mul64hi(Tp << z, den1 + 2 * __mul64hi(qs[0], B << 4)) +
+                            __mul64hi(Tm << z, den2 - 2 * __mul64hi(qs[1], A << 4));
+      out[g] = quot_s64(num, __umul64hi((unsigned long long)den1 << 3, (unsigned long long)den2 << 3), q + 1 + c - z);
     }
-  }
-#pragma unroll
-  for (int g = 0; g < NG; ++g) {  // S_g lies in [2^50, 2^63): no range check (see rcp_d)
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(den[g]));
-    const double e = fma(-den[g], y, K.one);
-    out[g] = K.mul(num[g], fma(y, fma(e, e, e), y));
     if (bad) out[g] = __longlong_as_double(0x7ff8000000000000LL);
   }
 }
