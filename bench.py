@@ -42,8 +42,11 @@ FP64_PEAK_TFLOPS = 2 * 2 * 152 * 2.07e9 / 1e12
 
 # ----------------------------------------------------------------------------- algorithmic work
 def stage_flops_per_cell(dim: int, pde: int, N: int, faces_per_cell: float = 2.0) -> dict:
-    """FP64 flops of one stage of Eq. (5) per cell, counted from the operations the split
-    stage evaluates (FMA = 2; add, multiply, reciprocal, square root = 1): the face pass
+    """FP64 flops of one stage of Eq. (5) per cell, counted from the operations of the split
+    stage with every sum in FP64 and every weight applied (FMA = 2; add, multiply, reciprocal,
+    square root = 1).  This is the work the rate is quoted on; the kernels need fewer FP64
+    instructions for it (sums relative to the outermost weight, the density's volume term
+    without quadrature, traces in fixed point on the integer pipes).  The face pass
     (two traces, the local Lax-Friedrichs flux at the N+1 face points, the projection on the
     transverse modes) for `faces_per_cell` faces, and the cell pass (sum-factorised volume
     term over symmetric Gauss pairs, lifting, stage combination averaged over the three
