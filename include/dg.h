@@ -213,7 +213,14 @@ dg_status dg_set_time(dg_mesh* m, const double* t);
 dg_status dg_get_time(dg_mesh* m, double* t);
 
 /* One full SSP-RK3 step: three times (stage, indicator, limiter), replayed from a CUDA
- * graph captured on the first call.  dt as in dg_rk_stage. */
+ * graph captured on the first call; in 1D with the TVB indicator, the CSWENO limiter and
+ * the positivity scaling off, one kernel does the whole step.  dt as in dg_rk_stage.
+ * Inside a caller's stream capture only that 1D step is supported (a step of another kind
+ * may be refused with DG_ECUDA: take dg_rk_stage, dg_flag_cells without host outputs, and
+ * the limiter calls there); dt must be the one in use already, since a new one is copied
+ * and waited for.  Captured calls work on the mesh's state at replay, also when direct
+ * calls ran in between; a mesh that has captured work pays a copy of the state per direct
+ * 1D step for it. */
 dg_status dg_step(dg_mesh* m, double dt, int indicator, double tvb_M);
 
 /* Largest characteristic speed over the cell means of each instance: out[2*i] (x) and

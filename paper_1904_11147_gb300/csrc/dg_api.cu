@@ -173,6 +173,7 @@ struct dg_mesh {
   Counters* cnt = nullptr;
   double* d_speed = nullptr;
   int cur = 0;          // buffer holding the current state
+  bool captured = false;  // a caller captured work on this mesh: the buffers keep their places (note_capture)
   int last_stage = 0;   // 0: state is u^n; s: output of stage s
   bool flags_valid = false;
   int limit_blocks = 0;
@@ -560,6 +561,18 @@ static L args(dg_mesh* m, int un, int us, int out) {
   return a;
 }
 
+// Work that a caller captured into a CUDA graph holds the addresses of U[0..2].  From the first
+// call inside a capture on, dg_step leaves every buffer where it is (see there), so that a
+// replay reads u^n and leaves its result where the next call looks for them, whatever ran
+// in between.  Called by every entry point whose work a capture can hold.
+static cudaError_t note_capture(dg_mesh* m) {
+  if (m->captured || !m->st) return cudaSuccess;  // (the legacy default stream cannot be captured)
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  const cudaError_t e = cudaStreamIsCapturing(m->st, &cs);
+  m->captured = cs != cudaStreamCaptureStatusNone;
+  return e;
+}
+
 // Times of the kBcDmr boundary data after stage s of SSP-RK3: the output of stage 1 holds at
 // t^n + dt, of stage 2 at t^n + dt/2, of stage 3 at t^n + dt, which becomes the new t^n.
 // kBcDmr meshes run the stage, the TVB indicator, the CSWENO limiter and the positivity
@@ -813,6 +826,7 @@ static void invalidate(dg_mesh* m) {
 extern "C" dg_status dg_set_modes(dg_mesh* m, const double* modes, size_t n, int is_device) {
   if (!m || !modes) return fail(DG_EINVAL, "null argument");
   if (n != mesh_doubles(m)) return fail(DG_EINVAL, "size %zu != mesh size %zu", n, mesh_doubles(m));
+  CK(note_capture(m));
   const double* src = modes;
   if (!is_device) {
     CK(cudaMemcpyAsync(m->lim, modes, n * sizeof(double), cudaMemcpyHostToDevice, m->st));
@@ -891,6 +905,7 @@ extern "C" dg_status dg_rk_stage(dg_mesh* m, int stage, double dt) {
     return fail(DG_ESTATE, "stage %d requested after stage %d", stage, m->last_stage);
   dg_status s = check_dt(m, dt);
   if (s != DG_OK) return s;
+  CK(note_capture(m));
   const int in = m->cur, out = stage_out(stage);
   k_stage(m, stage, in, out, dt > 0.0 ? dt : 0.0);
   CK(cudaGetLastError());
@@ -911,6 +926,7 @@ extern "C" dg_status dg_flag_cells(dg_mesh* m, int indicator, double tvb_M, int6
     return fail(DG_EINVAL, "unknown indicator %d", indicator);
   if (indicator == DG_IND_MLP && !m->has_mlp) return fail(DG_EINVAL, "no learned indicator attached to the mesh");
   if (!(tvb_M >= 0.0)) return fail(DG_EINVAL, "tvb_M must be >= 0");
+  CK(note_capture(m));
   if (indicator == DG_IND_MLP) {
     CK(learned_flags(m, tvb_M));
   } else if (indicator == DG_IND_KXRCF) {
@@ -940,6 +956,7 @@ extern "C" dg_status dg_flag_cells(dg_mesh* m, int indicator, double tvb_M, int6
 extern "C" dg_status dg_cswenolimit(dg_mesh* m) {
   if (!m) return fail(DG_EINVAL, "null mesh");
   if (!m->flags_valid) return fail(DG_ESTATE, "no troubled-cell flags for the current state");
+  CK(note_capture(m));
   if (m->use_b) CK(learned_limit(m));  // the learned flags, with their positivity fallback
   else k_limit(m);
   CK(cudaGetLastError());
@@ -952,6 +969,7 @@ extern "C" dg_status dg_parent_wenolimit(dg_mesh* m) {
   if (!m) return fail(DG_EINVAL, "null mesh");
   if (!m->flags_valid) return fail(DG_ESTATE, "no troubled-cell flags for the current state");
   if (m->min_side < m->N + 1) return fail(DG_EINVAL, "the parent WENO stencil needs %d cells per side", m->N + 1);
+  CK(note_capture(m));
   if (m->use_b) k_parent_list(m, m->lb_cell, m->lb_inst, m->cnt_b);
   else k_parent_list(m, m->list_cell, m->list_inst, m->cnt);
   CK(cudaGetLastError());
@@ -974,6 +992,7 @@ extern "C" dg_status dg_positivity_limit(dg_mesh* m, double eps0) {
   if (!m) return fail(DG_EINVAL, "null mesh");
   if (m->pde != DG_EULER) return fail(DG_EINVAL, "the positivity-preserving scaling is defined for the Euler equations");
   if (!(eps0 > 0.0) || !std::isfinite(eps0)) return fail(DG_EINVAL, "eps0 must be positive and finite");
+  CK(note_capture(m));
   k_pp(m, eps0);
   CK(cudaGetLastError());
   m->flags_valid = false;
@@ -1119,20 +1138,18 @@ extern "C" dg_status dg_step(dg_mesh* m, double dt, int indicator, double tvb_M)
     dg_status s = check_dt(m, dt);
     if (s != DG_OK) return s;
   }
+  CK(note_capture(m));
   m->cur = 0;
   if (m->dim == 1 && indicator == DG_IND_TVB && m->limiter == DG_LIM_CSWENO && !m->pp_on) {
-    // the whole step in one kernel, u^n to the next buffer; the buffers then change places.
-    // Inside a caller's stream capture the recorded work must not depend on the replay's
-    // number: there the result is copied back instead.
+    // the whole step in one kernel, u^n to the next buffer; the buffers then change places, on
+    // a mesh with work in a caller's capture the result is copied back instead.
     LaunchArgs a = args<LaunchArgs>(m, 0, 0, 1);
     a.tiles = m->d_step_tiles;
     a.ntiles = m->n_step_tiles;
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (m->st) CK(cudaStreamIsCapturing(m->st, &cs));
     launch_step1(m->pde, m->N, a, tvb_M, m->flag_totals);
     CK(cudaGetLastError());
     m->launches++;
-    if (cs != cudaStreamCaptureStatusNone) {
+    if (m->captured) {
       CK(cudaMemcpyAsync(m->U[0], m->U[1], sizeof(double) * m->ctot * m->V * m->NP, cudaMemcpyDeviceToDevice, m->st));
     } else {
       std::swap(m->U[0], m->U[1]);
@@ -1537,6 +1554,7 @@ extern "C" dg_status dg_indicator_logits(dg_mesh* m, float* logits) {
   if (m && m->bc == DG_BC_DMR) return fail(DG_EINVAL, "not available with the double Mach reflection boundaries");
   if (!m || !logits) return fail(DG_EINVAL, "null argument");
   if (!m->has_mlp) return fail(DG_EINVAL, "no learned indicator attached to the mesh");
+  CK(note_capture(m));
   CK(cudaMemsetAsync(m->cnt, 0, sizeof(Counters), m->st));
   k_flag_learned(m, logits);
   CK(cudaGetLastError());
@@ -1557,6 +1575,7 @@ extern "C" dg_status dg_refined_arith(int op, const double* x, double* out, int6
 extern "C" dg_status dg_harvest(dg_mesh* m, double tvb_M, float* X, uint8_t* flags, float* change) {
   if (m && m->bc == DG_BC_DMR) return fail(DG_EINVAL, "not available with the double Mach reflection boundaries");
   if (!m || !X || !flags || !change) return fail(DG_EINVAL, "null argument");
+  CK(note_capture(m));
   LaunchArgs a = args<LaunchArgs>(m, 0, m->cur, m->cur);
   const double c0 = mean_factor(m);
   m->use_b = false;
