@@ -535,6 +535,7 @@ __device__ __noinline__ int tvb_cell(const double* __restrict__ U, const Inst& I
 //     the FP64 means and difference to 2^-52 |m|.  Margin 2^-21 |d| + 2^-44 max |m|.
 //   - every margin also holds 2^-100 for parts below the float range; infinities and NaN
 //     satisfy none of the comparisons below.
+//   - a value above mhi >= 0 with its margin has a known sign.
 // A test is decided when its comparisons hold with the margins and the windows of
 // tvb_changes_bits (2^-37 relative, 2^-39 of the largest magnitude) to spare: then the FP64
 // test decides the same and is not near a threshold.
@@ -633,8 +634,11 @@ __global__ void __launch_bounds__(256)
   if (active) {
     // the double Mach reflection's ghosts are left to FP64
     if (bc == kBcDmr && (ix == 0 || iy == 0 || ix == I.nx - 1 || iy == I.ny - 1)) fl = 2;
-    const float xlo = s_mh2[0] * (1.0f - 0x1p-20f), xhi = fmaf(s_mh2[0], 1.0f + 0x1p-20f, 0x1p-100f);
-    const float ylo = s_mh2[1] * (1.0f - 0x1p-20f), yhi = fmaf(s_mh2[1], 1.0f + 0x1p-20f, 0x1p-100f);
+    // (a negative M, which dg_step and dg_harvest take: mlo is not met then, and mhi must not
+    // fall below 0, or a sign that the margin leaves open would count as known)
+    const float xlo = s_mh2[0] * (1.0f - 0x1p-20f), ylo = s_mh2[1] * (1.0f - 0x1p-20f);
+    const float xhi = s_mh2[0] < 0.0f ? 0x1p-100f : fmaf(s_mh2[0], 1.0f + 0x1p-20f, 0x1p-100f);
+    const float yhi = s_mh2[1] < 0.0f ? 0x1p-100f : fmaf(s_mh2[1], 1.0f + 0x1p-20f, 0x1p-100f);
 #pragma unroll
     for (int v = 0; v < V; ++v) {
       const double* P = U + (long long)(v * NP) * ctot + g;
