@@ -372,13 +372,21 @@ dg_status dg_cswenolimit_noalloc(int dim, int pde, int N, int nx, int ny, const 
                                  double tvb_M, const double* u_in, double* u_out, int64_t* n_flagged, int64_t* n_near,
                                  void* stream);
 
-/* The refined arithmetic of the FP64 kernels (not part of the method): op 0 the reciprocal,
- * op 1 the square root, as the 2D Euler fluxes and the WENO weights evaluate them -- the
- * hardware's approximation refined by one Householder step of order three, within one or
- * two ulps of the IEEE results; arguments outside the refined range (zero, subnormal,
- * |x| >= 2^1022, inf, NaN, and non-positive square-root arguments) give the IEEE result.
- * x and out are device arrays of n doubles; asynchronous on stream.  For checking that
- * arithmetic against IEEE operations.  Errors: DG_EINVAL, DG_ECUDA. */
+/* The kernels' own arithmetic (not part of the method), for checking it against IEEE operations and
+ * exact values:
+ *   op 0, 1  reciprocal and square root of the fused 2D stage and of the limiters' eigenvectors
+ *   op 2, 3  the same as the split 2D stage (the default) and the 1D kernels evaluate them
+ *   op 4     the 2D limiters' quotient t / s 2^q, rounded to nearest (the value before rounding within
+ *            2^-60); out of the normal range: 0 or infinity.  x: three planes of n 64-bit integers, t
+ *            (signed), s (unsigned, not 0), q.
+ *   op 5     t 2^q rounded to nearest; x: two planes, t and q
+ *   op 6..8  the split stage's fixed-point traces for N = op - 5: x holds NP planes of n modes, out N+1
+ *            planes with twice the trace on the east face at its N+1 Gauss points
+ * Ops 0 to 3 are the hardware's approximation refined by one Householder step of order three, within
+ * one or two ulps of the IEEE results; arguments outside the refined range (zero, subnormal,
+ * |x| >= 2^1022 (reciprocal), inf, NaN, and non-positive square-root arguments) give the IEEE
+ * result.  x and out are device arrays (n doubles, or planes of n); asynchronous on stream.
+ * Errors: DG_EINVAL, DG_ECUDA. */
 dg_status dg_refined_arith(int op, const double* x, double* out, int64_t n, void* stream);
 
 /* Thread-local text of the last error (never NULL). */

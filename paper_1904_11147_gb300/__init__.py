@@ -316,9 +316,12 @@ class Mesh:
 
 
 def refined_arith(op, x, out, stream=0):
-    """dg_refined_arith on CUDA float64 tensors: op 0 reciprocal, 1 square root."""
+    """dg_refined_arith on CUDA tensors of 8-byte elements (op 0 and 2 reciprocal, 1 and 3 square
+    root; 4 quotient, 5 rounding, 6..8 traces on planes: x [planes][n])."""
+    planes = {4: 3, 5: 2, 6: 3, 7: 6, 8: 10}.get(int(op), 1)
+    assert x.numel() % planes == 0 and out.numel() >= (op - 4 if op >= 6 else 1) * (x.numel() // planes)
     _check(lib().dg_refined_arith(int(op), ctypes.c_void_p(x.data_ptr()), ctypes.c_void_p(out.data_ptr()),
-                                  x.numel(), ctypes.c_void_p(int(stream))))
+                                  x.numel() // planes, ctypes.c_void_p(int(stream))))
     return out
 
 

@@ -13,6 +13,7 @@
 
 #include "../../include/dg.h"
 #include "dg_shared.cuh"
+#include "dg_weno.cuh"
 #include "tables.h"
 
 namespace dg {
@@ -23,6 +24,7 @@ cudaError_t prepare2(int pde, int N);
 cudaError_t upload_tables_stage2(const dgt::Tabs* tabs);
 cudaError_t prepare_stage2_split(int pde, int N);
 int face_chunk2();
+void launch_trace_probe(cudaStream_t st, int N, const double* x, double* out, long long n, int nblocks);
 int cell_chunk2();
 int tile_w1();
 int step_tile1();
@@ -765,11 +767,22 @@ static __global__ void k_flag_bit0(const unsigned char* __restrict__ in, unsigne
     out[g] = in[g] & 1;
 }
 
-// The refined reciprocal (op 0) and square root (op 1) the Euler fluxes and the WENO
-// weights use, on a device array (dg_refined_arith).
-static __global__ void k_refined_arith(int op, const double* __restrict__ x, double* __restrict__ out, long long n) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    out[i] = op == 0 ? rcp_d(x[i]) : sqrt_d(x[i]);
+// The kernels' own arithmetic on a device array (dg_refined_arith): rcp_d, sqrt_d (op 0, 1: fused stage,
+// limiters' eigenvectors), rcp_k, sqrt_t (2, 3: split 2D stage, 1D), quot_s64 (4) and pack_s64 (5) on
+// planes of 64-bit integers.
+static __global__ void k_refined_arith(int op, const double* __restrict__ x, double* __restrict__ out, long long n,
+                                       Reg64 K) {
+  const long long* k = reinterpret_cast<const long long*>(x);
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    double r;
+    if (op == 0) r = rcp_d(x[i]);
+    else if (op == 1) r = sqrt_d(x[i]);
+    else if (op == 2) r = rcp_k(x[i], K);
+    else if (op == 3) r = sqrt_t(x[i], K, 0.375, 0.5);
+    else if (op == 4) r = quot_s64(k[i], (unsigned long long)k[n + i], (int)k[2 * n + i]);
+    else r = pack_s64(k[i], (int)k[n + i]);
+    out[i] = r;
+  }
 }
 
 // ----------------------------------------------------------------------------- layout
@@ -1564,10 +1577,17 @@ extern "C" dg_status dg_indicator_logits(dg_mesh* m, float* logits) {
 }
 
 extern "C" dg_status dg_refined_arith(int op, const double* x, double* out, int64_t n, void* stream) {
-  if ((op != 0 && op != 1) || !x || !out || n < 0) return fail(DG_EINVAL, "bad arguments");
+  if (op < 0 || op > 8 || !x || !out || n < 0) return fail(DG_EINVAL, "bad arguments");
   if (n == 0) return DG_OK;
   const cudaStream_t st = (cudaStream_t)stream;
-  k_refined_arith<<<(int)std::min<long long>((n + 255) / 256, 65535), 256, 0, st>>>(op, x, out, n);
+  const int nb = (int)std::min<long long>((n + 255) / 256, 65535);
+  if (op >= 6) {
+    const dg_status s = dg_ensure_tables_internal();
+    if (s != DG_OK) return s;
+    launch_trace_probe(st, op - 5, x, out, n, nb);
+  } else {
+    k_refined_arith<<<nb, 256, 0, st>>>(op, x, out, n, Reg64{1.0, -0.0});
+  }
   CK(cudaGetLastError());
   return DG_OK;
 }

@@ -51,7 +51,8 @@ __device__ __forceinline__ double neg_if(double x, bool f) {
   return __longlong_as_double(__double_as_longlong(x) ^ (long long)((unsigned long long)f << 63));
 }
 
-// Reciprocal and square root of the 2D Euler stage fluxes and of the WENO weights, from
+// Reciprocal and square root of the fused 2D stage's fluxes, the limiters' eigenvectors and the 1D
+// parent limiter's weights (the split stage and 1D have their own forms, rcp_k and sqrt_t), from
 // the hardware's ~20-bit approximations refined by one step of Householder's third-order
 // iteration: with e the relative error of the seed y, 1/x = y / (1 - e) and
 // 1/sqrt(x) = y (1 - e)^(-1/2), and the first three terms of those series,

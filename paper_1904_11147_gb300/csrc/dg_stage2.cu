@@ -515,6 +515,20 @@ __global__ void __launch_bounds__(kCellChunk, (PDE == 1 && N == 3) ? 1 : 2)
   }
 }
 
+// The traces alone (dg_refined_arith): out[q][i] from the modes x[m][i], i < n.
+template <int N>
+__global__ void __launch_bounds__(256) k_trace_probe(const double* __restrict__ x, double* __restrict__ out, long long n) {
+  using T = STab<N>;
+  __shared__ __align__(16) double tab[T::FACE];
+  if (threadIdx.x < T::XF) tab[threadIdx.x] = g_stab[N - 1][threadIdx.x];
+  __syncthreads();
+  for (long long i = blockIdx.x * 256ll + threadIdx.x; i < n; i += gridDim.x * 256ll) {
+    const TraceVal<N> o = trace<N>(x + i, n, 0, false, false, false, nullptr, reinterpret_cast<const long long*>(tab));
+#pragma unroll
+    for (int q = 0; q <= N; ++q) out[q * n + i] = o.v[q];
+  }
+}
+
 // dynamic shared memory of the cell pass: the modes of its 256 cells
 constexpr size_t cell_smem(int pde, int N) {
   return smem_modes(pde, N) ? sizeof(long long) * 4 * ((N + 1) * (N + 2) / 2) * kCellChunk : 0;
@@ -546,6 +560,12 @@ cudaError_t prepare_stage2_split(int pde, int N) {
   const int bytes = (int)st2::cell_smem(pde, N);
   return N == 2 ? cudaFuncSetAttribute(st2::k_cell2<1, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)
                 : cudaFuncSetAttribute(st2::k_cell2<1, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
+
+void launch_trace_probe(cudaStream_t st, int N, const double* x, double* out, long long n, int nblocks) {
+  if (N == 1) st2::k_trace_probe<1><<<nblocks, 256, 0, st>>>(x, out, n);
+  else if (N == 2) st2::k_trace_probe<2><<<nblocks, 256, 0, st>>>(x, out, n);
+  else st2::k_trace_probe<3><<<nblocks, 256, 0, st>>>(x, out, n);
 }
 
 int face_chunk2() { return st2::kFaceChunk; }
