@@ -70,16 +70,13 @@ void pack(const dgt::Tabs& t, double* h) {
   h[S::NZ] = -0.0;
   h[S::C38] = 0.375;
   h[S::HALF] = 0.5;
-  auto put = [&](int k, double v) {
-    const long long i = std::llrint(v);
-    std::memcpy(h + k, &i, sizeof(i));
-  };
+  auto put = [&](int k, long long i) { std::memcpy(h + k, &i, sizeof(i)); };
   auto wp = [&](int q, int b) { return t.gw[q] * t.psi_q[q][b]; };
   auto wd = [&](int q, int b) { return t.gw[q] * t.dpsi_q[q][b]; };
   for (int n = 0; n < N1; ++n) {
-    put(S::KP1 + n, std::ldexp(t.kp1[n], 61));
+    put(S::KP1 + n, t.kp1_fix[n]);
     for (int q = 0; q < NX; ++q) {
-      put(S::KQ + q * N1 + n, std::ldexp(t.kq[q][n], 62));
+      put(S::KQ + q * N1 + n, t.kq_fix[q][n]);
       h[S::KD + q * N1 + n] = t.kq[q][n];
     }
     h[S::KAP + n] = wp(1, n) / wp(0, n);
@@ -154,20 +151,23 @@ __device__ __noinline__ TraceVal<N> trace(const double* __restrict__ p, long lon
     if (cst) x = m == 0 ? 2.0 * *cst : 0.0;  // constant state: U_00 = 2 mean, no other mode
     u[m] = neg_if(x, ((fn && (n & 1)) != (ft && (t & 1))) != wall);
   }
-  // sums over the normal degree (an eighth; sum |KP1| < 8), then at the points (a quarter)
+  // sums over the normal degree in units of 8 X, then at the points.  Below 2^62.5 all of them: X
+  // below 2^63, 2^62, 2^61, sum_t |KQ_t| sum_{n <= N-t} |KP1_n| = 3.7, 9.5, 19.6 and 4 |e_1| / |X| at most
+  // 1/2, 1.37, 2.49 for N = 1, 2, 3.
+  constexpr int F = 11 - N;
   long long X[NP], e[N1], val[Q];
-  const int E = align_modes<NP>(u, X);
+  const int E = align_modes<NP, F, 3>(u, X);
 #pragma unroll
   for (int t = 0; t <= N; ++t) {
     long long z = X[mode_idx(0, t)] >> 3;
 #pragma unroll
-    for (int n = 1; n <= N - t; ++n) z += __mul64hi(itab[T::KP1 + n], X[mode_idx(n, t)]);
+    for (int n = 1; n <= N - t; ++n) z += mul_rn(itab[T::KP1 + n], X[mode_idx(n, t)]);
     e[t] = z;
   }
   eval_fix<N>(e, itab + T::KQ, val);
 #pragma unroll
   for (int q = 0; q < Q; ++q)
-    o.v[q] = E < 2047 ? pack_s64(val[q], E - 1079) : __longlong_as_double(0x7ff8000000000000LL);
+    o.v[q] = E < 2047 ? pack_s64<true>(val[q], E - 1072 - F) : __longlong_as_double(0x7ff8000000000000LL);
   return o;
 }
 
@@ -331,7 +331,7 @@ __global__ void __launch_bounds__(kCellChunk, (PDE == 1 && N == 3) ? 1 : 2)
       u[m] = __ldg(us + (long long)(v * NP + m) * ctot + g);
       X[m] = __double_as_longlong(u[m]);
     }
-    if constexpr (kFix) E[v] = align_modes<NP>(u, X);
+    if constexpr (kFix) E[v] = align_modes<NP, 8, 2>(u, X);  // |X| < 2^61; sums below 2^62, 4 |tb_1| below 2^62.3
 #pragma unroll
     for (int m = 0; m < NP; ++m) {
       if constexpr (kSmemU) s_x[(v * NP + m) * kCellChunk + threadIdx.x] = X[m];
@@ -390,22 +390,22 @@ __global__ void __launch_bounds__(kCellChunk, (PDE == 1 && N == 3) ? 1 : 2)
 #pragma unroll
       for (int v = 0; v < V; ++v) {
         if constexpr (kFix) {
-          // x sums over psi_0 at -x_p (side 0) or x_p, a quarter (formed again for each side: the
+          // x sums over psi_0 at -x_p (side 0) or x_p in units of 4 X (formed again for each side: the
           // integer pipes have the time, the registers are short), then the y points
           const long long* c = itab + T::KQ + p * N1;
           long long tb[N1], val[Q];
   #pragma unroll
           for (int b = 0; b <= N; ++b) {
             long long ev = x(v, mode_idx(0, b)) >> 2, od = 0;
-            if (N - b >= 2) ev += __mul64hi(c[N >= 2 ? 2 : 0], x(v, mode_idx(N - b >= 2 ? 2 : 0, b)));
-            if (!mid && b < N) od = __mul64hi(c[1], x(v, mode_idx(b < N ? 1 : 0, b)));
-            if (N - b >= 3) od += __mul64hi(c[3 <= N ? 3 : 0], x(v, mode_idx(N - b >= 3 ? 3 : 0, b)));
+            if (N - b >= 2) ev += mul_rn(c[N >= 2 ? 2 : 0], x(v, mode_idx(N - b >= 2 ? 2 : 0, b)));
+            if (!mid && b < N) od = mul_rn(c[1], x(v, mode_idx(b < N ? 1 : 0, b)));
+            if (N - b >= 3) od += mul_rn(c[3 <= N ? 3 : 0], x(v, mode_idx(N - b >= 3 ? 3 : 0, b)));
             tb[b] = side == 0 ? ev + od : ev - od;
           }
           eval_fix<N>(tb, itab + T::KQ, val);
   #pragma unroll
           for (int q = 0; q < Q; ++q)
-            col[v][q] = E[v] < 2047 ? pack_s64(val[q], E[v] - 1080) : __longlong_as_double(0x7ff8000000000000LL);
+            col[v][q] = E[v] < 2047 ? pack_s64<true>(val[q], E[v] - 1081) : __longlong_as_double(0x7ff8000000000000LL);
         } else {
           eval_gauss2<N>(tb[side][v], tab + T::KD, K, col[v]);
         }
