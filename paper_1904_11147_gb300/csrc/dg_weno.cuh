@@ -83,21 +83,22 @@ __device__ __forceinline__ double pack_s64(long long t, int q) {
   return __longlong_as_double((long long)(bits | ((unsigned long long)t & 0x8000000000000000ull)));
 }
 
-// X[m] 2^(E - 1075 - F) = u[m], |X| < 2^(53 + F); values 2^-(53 + F) below the largest are dropped, and
-// so are numbers below 2^-958.  The low LOW bits of the modes of degree 0 in the first
-// direction are cleared: those enter the sums shifted by LOW.  E >= 2047: a mode is not finite.
+// X[m] 2^(E - 1075 - F) = u[m], |X| < 2^(53 + F); values 2^-(53 + F) below the largest are dropped.  The
+// low LOW bits of the modes of degree 0 in the first direction are cleared: those enter the
+// sums shifted by LOW.  E >= 2047: a mode is not finite.
 template <int M, int F, int LOW>
 __device__ __forceinline__ int align_modes(const double (&u)[M], long long (&X)[M]) {
-  unsigned top = 64u << 20;
+  unsigned top = 1u << 20;
 #pragma unroll
   for (int m = 0; m < M; ++m) top = max(top, (unsigned)__double2hiint(u[m]) & 0x7fffffffu);
   const int E = (int)(top >> 20);
 #pragma unroll
   for (int m = 0; m < M; ++m) {
-    const unsigned hi = (unsigned)__double2hiint(u[m]), lo = (unsigned)__double2loint(u[m]);
-    const unsigned long long w = ((unsigned long long)__funnelshift_l(lo, (hi & 0xfffffu) | 0x100000u, F) << 32) | (lo << F);
+    const unsigned hi = (unsigned)__double2hiint(u[m]), lo = (unsigned)__double2loint(u[m]), ex = (hi >> 20) & 0x7ffu;
+    const unsigned sig = (hi & 0xfffffu) | (min(ex, 1u) << 20);  // (no leading 1 below the normal range)
+    const unsigned long long w = ((unsigned long long)__funnelshift_l(lo, sig, F) << 32) | (lo << F);
     const unsigned long long keep = mode_a(m) == 0 ? ~((1ull << LOW) - 1) : ~0ull;
-    const long long x = (long long)((w >> min(E - (int)((hi >> 20) & 0x7ffu), 63)) & keep), s = (long long)((int)hi >> 31);
+    const long long x = (long long)((w >> min(E - (int)max(ex, 1u), 63)) & keep), s = (long long)((int)hi >> 31);
     X[m] = (x ^ s) - s;
   }
   return E;
