@@ -43,13 +43,21 @@ __device__ __forceinline__ int reflect(int j, int n, int bc) {
 // the sums that no average needs left out, the subcell averages take 90 (P2) of the 650 FP64
 // instructions a lane spent on a troubled cell less (1024^2 P2 step 11.1 -> 10.8 ms, P3 batch of 8 x
 // 128 x 512 cells 30.0 -> 28.4 ms).  Numbers within a binade of the largest and the
-// smallest normal ones, and non-finite ones, stay as they are.
+// smallest normal ones, and non-finite ones, stay as they are: an error of 2^-1021 at most at the
+// lower end (see kSmall); at the upper one the smoothness indicators overflow anyway.
 __device__ __forceinline__ double exp_add(double x, int d) {
   const unsigned hi = (unsigned)__double2hiint(x), ex = (hi & 0x7ff00000u) - 0x00200000u;
   return __hiloint2double((int)(ex <= 0x7fb00000u ? hi + (unsigned)(d << 20) : hi), __double2loint(x));
 }
 __device__ __forceinline__ double dbl(double x) { return exp_add(x, 1); }
 __device__ __forceinline__ double half(double x) { return exp_add(x, -1); }
+
+// A cell whose data all lie below 2^-959 (exponent word below kSmall) is limited on them times 2^500:
+// neither the halves above nor the reconstruction's quotients are exact down there.  The limiter commutes with the factor, since the smoothness indicators are
+// far below eps either way.  The two steps it takes are functions that no other cell calls
+// (multiplying in place under a condition took 5 to 8 % of the limiter's time).
+constexpr unsigned kSmall = 64u << 20;
+constexpr double kSmallUp = 0x1p500;
 
 // Where the averages of one troubled cell and one variable go: the 2N x differences of row
 // ky (item k between averages k and k + 1) and the row's middle average.
@@ -58,9 +66,9 @@ __device__ __forceinline__ double half(double x) { return exp_add(x, -1); }
 // CSWENO: subcell averages of the 3 x 3 neighbourhood.  A neighbour's modes, mirrored in x on
 // the right side, give per transverse degree b the N - 1 differences inside it and the
 // average next to the troubled cell; the y part then gives them for its N rows.
-// Returns the largest exponent word of the modes that no average needs: the averages of a
-// non-finite state must stay non-finite whichever mode holds it.
-template <int N, class Dst>
+// Returns the largest exponent word of the modes: the averages of a non-finite state must stay
+// non-finite whichever mode holds it.  SMALL: the modes times 2^500.
+template <int N, bool SMALL, class Dst>
 __device__ __forceinline__ unsigned subcell_diffs(const double* __restrict__ U, long long ctot, const Inst& I, int inst,
                                                   int ix, int iy, int v, int bc, const double* __restrict__ bcd,
                                                   const double* __restrict__ tab, const Reg64& K, Dst dst) {
@@ -103,6 +111,7 @@ __device__ __forceinline__ unsigned subcell_diffs(const double* __restrict__ U, 
     for (int m = 0; m < NP; ++m) {
       double x = __ldg(p + (long long)m * ctot);
       if (cst) x = m == 0 ? 2.0 * cst[v] : 0.0;
+      if constexpr (SMALL) x *= kSmallUp;
       u[m] = neg_if(x, ((mx && (mode_a(m) & 1)) != (fy && (mode_b(m) & 1))) != fv);
     }
 #pragma unroll
@@ -178,10 +187,12 @@ __device__ __forceinline__ unsigned subcell_diffs(const double* __restrict__ U, 
 }
 
 // Parent WENO: means of the whole cells (ix - N .. ix + N) x (iy - N .. iy + N).
-template <int N, class Dst>
-__device__ __forceinline__ void cell_diffs(const double* __restrict__ U, long long ctot, const Inst& I, int ix, int iy,
-                                           int v, int bc, const double* __restrict__ tab, const Reg64& K, Dst dst) {
+template <int N, bool SMALL, class Dst>
+__device__ __forceinline__ unsigned cell_diffs(const double* __restrict__ U, long long ctot, const Inst& I, int ix,
+                                               int iy, int v, int bc, const double* __restrict__ tab, const Reg64& K,
+                                               Dst dst) {
   using L = LimTab<N>;
+  unsigned top = 0;
   const double* p = U + (long long)(v * np_of(2, N)) * ctot + I.off;
   const double p0 = tab[L::P0];
 #pragma unroll 1
@@ -190,12 +201,41 @@ __device__ __forceinline__ void cell_diffs(const double* __restrict__ U, long lo
     double prev = 0.0;
 #pragma unroll
     for (int kx = 0; kx < 2 * N + 1; ++kx) {
-      const double a = K.mul(K.mul(__ldg(row + reflect(ix + kx - N, I.nx, bc)), p0), p0);
+      double x = __ldg(row + reflect(ix + kx - N, I.nx, bc));
+      if constexpr (SMALL) x *= kSmallUp;
+      top = max(top, (unsigned)__double2hiint(x) & 0x7fffffffu);
+      const double a = K.mul(K.mul(x, p0), p0);
       if (kx) dst.diff(ky, kx - 1) = K.sub(a, prev);
       if (kx == N) dst.mid(ky) = a;
       prev = a;
     }
   }
+  return top;
+}
+
+// The differences of listed cell g, variable v
+template <int N, bool PARENT, bool SMALL, class Dst>
+__device__ __forceinline__ unsigned stencil_diffs(const double* __restrict__ U, const Inst* __restrict__ insts,
+                                                  long long ctot, int bc, long long g, int inst, int v,
+                                                  const double* __restrict__ bcd, const double* __restrict__ tab,
+                                                  const Reg64& K, Dst dst) {
+  const Inst I = insts[inst];
+  const int loc = (int)(g - I.off);
+  const int ix = loc % I.nx, iy = loc / I.nx;
+  if constexpr (PARENT) return cell_diffs<N, SMALL>(U, ctot, I, ix, iy, v, bc, tab, K, dst);
+  else return subcell_diffs<N, SMALL>(U, ctot, I, inst, ix, iy, v, bc, bcd, tab, K, dst);
+}
+template <int N, bool PARENT, class Dst>
+__device__ __noinline__ void stencil_diffs_small(const double* __restrict__ U, const Inst* __restrict__ insts,
+                                                 long long ctot, int bc, long long g, int inst, int v,
+                                                 const double* __restrict__ bcd, const double* __restrict__ tab, Dst dst) {
+  const Reg64 K{tab[LimTab<N>::ONE], tab[LimTab<N>::NZ]};
+  stencil_diffs<N, PARENT, true>(U, insts, ctot, bc, g, inst, v, bcd, tab, K, dst);
+}
+// the limited modes 1..NP-1 of a variable back to their size
+template <int N>
+__device__ __noinline__ void unscale_small(double* __restrict__ lim, long long cap) {
+  for (int m = 1; m < np_of(2, N); ++m) lim[m * cap] *= 1.0 / kSmallUp;
 }
 
 // Eigenvector products of the 2D Euler flux Jacobian at the troubled cell's mean state,
@@ -318,18 +358,11 @@ __global__ void __launch_bounds__(kQuadThreads, quad_blocks(N))
     const long long g = list_cell[i];
     const int inst = list_inst[i];
     Eig e;
-    bool bad = false;
-    {
-      const Inst I = insts[inst];
-      const int loc = (int)(g - I.off);
-      const int ix = loc % I.nx, iy = loc / I.nx;
-      if constexpr (PARENT) {
-        cell_diffs<N>(U, ctot, I, ix, iy, q, bc, tab, K, Dst{S, q});
-      } else {
-        const unsigned top = subcell_diffs<N>(U, ctot, I, inst, ix, iy, q, bc, bcd, tab, K, Dst{S, q});
-        bad = __any_sync(0xfu << (lane & ~3), top >= 0x7ff00000u);
-      }
-    }
+    const unsigned quad = 0xfu << (lane & ~3);
+    const unsigned top = stencil_diffs<N, PARENT, false>(U, insts, ctot, bc, g, inst, q, bcd, tab, K, Dst{S, q});
+    const bool bad = !PARENT && __any_sync(quad, top >= 0x7ff00000u);
+    const bool small = __all_sync(quad, top < kSmall);
+    if (small) stencil_diffs_small<N, PARENT>(U, insts, ctot, bc, g, inst, q, bcd, tab, Dst{S, q});
     __syncwarp();
     {
       double m[4];
@@ -428,6 +461,7 @@ __global__ void __launch_bounds__(kQuadThreads, quad_blocks(N))
         if (active) lim[(long long)(q * NP + mode_idx(a, b)) * cap + i] = s;
       }
     }
+    if (small && active) unscale_small<N>(lim + (long long)(q * NP) * cap + i, cap);
     __syncwarp();  // the next cell's averages overwrite the items
   }
 }
@@ -462,14 +496,9 @@ __global__ void __launch_bounds__(kCellThreads)
   for (unsigned int i = blockIdx.x * kCellThreads + threadIdx.x; i < n; i += gridDim.x * kCellThreads) {
     const long long g = list_cell[i];
     const int inst = list_inst[i];
-    unsigned top = 0;
-    {
-      const Inst I = insts[inst];
-      const int loc = (int)(g - I.off);
-      const int ix = loc % I.nx, iy = loc / I.nx;
-      if constexpr (PARENT) cell_diffs<N>(U, ctot, I, ix, iy, 0, bc, tab, K, A);
-      else top = subcell_diffs<N>(U, ctot, I, inst, ix, iy, 0, bc, nullptr, tab, K, A);
-    }
+    const unsigned top = stencil_diffs<N, PARENT, false>(U, insts, ctot, bc, g, inst, 0, nullptr, tab, K, A);
+    const bool bad = !PARENT && top >= 0x7ff00000u, small = top < kSmall;
+    if (small) stencil_diffs_small<N, PARENT>(U, insts, ctot, bc, g, inst, 0, nullptr, tab, A);
 #pragma unroll 1
     for (int ky = 0; ky < NS; ++ky) {
       double d[2 * N], r[NG];
@@ -516,7 +545,8 @@ __global__ void __launch_bounds__(kCellThreads)
     }
 #pragma unroll
     for (int m = 1; m < NP; ++m)
-      lim[(long long)m * cap + i] = top >= 0x7ff00000u ? __longlong_as_double(0x7ff8000000000000LL) : acc[m];
+      lim[(long long)m * cap + i] = bad ? __longlong_as_double(0x7ff8000000000000LL) : acc[m];
+    if (small) unscale_small<N>(lim + i, cap);
   }
 }
 

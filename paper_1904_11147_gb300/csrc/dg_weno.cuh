@@ -263,6 +263,8 @@ __device__ __forceinline__ double quot_s64(long long t, unsigned long long s, in
 //         to theirs.  A term loses at most 2^-62 of the largest one, and every product at most
 //         one unit of the sum, half of it on average (added back at the start).
 //   u_g - avg[N] = T_g / S_g, in integers rounded once, or in FP64
+// Out of FP64's normal range: subnormal differences enter with their leading zeros; a quotient in
+// integers below 2^-1022 is 0 (see kSmall in dg_limit2.cu).
 // FP64 instructions per call: 2 / 12 / 32 for N = 1, 2, 3 (10 / 27 / 64 with the quotient in
 // FP64, 20 / 71 / 142 with all of it), next to some 250 / 800 / 1,700 integer ones.  From all of it
 // in FP64 to FP64 quotients: limiter of 130k P2 cells 974 -> 730 us, of 140k P3 cells 2,200 ->
@@ -330,8 +332,8 @@ __device__ __forceinline__ void weno_diff(const double (&d)[2 * N], const double
     const unsigned hi = (unsigned)__double2hiint(d[k]), ab = hi & 0x7fffffffu;
     bad = bad || ab >= 0x7ff00000u;
     neg |= (hi >> 31) << k;
-    dm[k] = unpack_pos(__hiloint2double((int)ab, __double2loint(d[k])));
-    if (ab < 0x00100000u) dm[k] = U64f{0ull, -(1 << 20)};  // zero (or subnormal)
+    const unsigned lo = (unsigned)__double2loint(d[k]), one = ab >= 0x00100000u ? 0x80000000u : 0u;
+    dm[k] = U64f{((unsigned long long)(__funnelshift_l(lo, ab, 11) | one) << 32) | (lo << 11), (int)max(ab >> 20, 1u)};
   }
   U64f X[N1][N];
   int ex = -(1 << 20), ep = P[0].e;
