@@ -259,9 +259,10 @@ __device__ __forceinline__ double quot_s64(long long t, unsigned long long s, in
 //         stencils' squares, as U64f (any magnitude of the data)
 //   X_ij  P_i d_{i+j}, sign apart
 //   T_g, S_g   sum wc X and sum wh P in 64-bit fixed point: all X are shifted to the largest
-//         one's exponent (below 2^62, so a sum of |wc| / 4 < 1/4 each stays below 2^63), all P
-//         to theirs.  A term loses at most 2^-62 of the largest one, and every product at most
-//         one unit of the sum, half of it on average (added back at the start).
+//         one's exponent (below 2^62), all P to theirs.  With sum |wc| <= 4.7 (below 8) and sum wh <=
+//         3.7 (below 4) per point both stay below 2^63 (dgt::sums_fit).  A term loses at most 2^-62
+//         of the largest one, and every product at most one unit of the sum, half of it on
+//         average (added back at the start).
 //   u_g - avg[N] = T_g / S_g, in integers rounded once, or in FP64
 // Out of FP64's normal range: subnormal differences enter with their leading zeros; a quotient in
 // integers below 2^-1022 is 0 (see kSmall in dg_limit2.cu).

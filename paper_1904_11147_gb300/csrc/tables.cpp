@@ -133,6 +133,24 @@ void primitive_deriv_rows(int n, const ld* e, int l, ld x, ld* w) {
 
 }  // namespace
 
+bool sums_fit(const Tabs& t, bool parent) {
+  for (int g = 0; g < t.NG; ++g) {
+    double c[2] = {0, 0}, h[2] = {0, 0};  // all stencils but the one with a negative weight; that one
+    for (int i = 0; i <= t.N; ++i) {
+      const int k = i == weno_neg(t.N, g, parent);
+      if (!(t.wh[g][i] < 2.0)) return false;
+      h[k] += t.wh[g][i];
+      for (int j = 0; j < t.N; ++j) {
+        if (!(std::fabs(t.wc[g][i][j]) < 2.0)) return false;
+        c[k] += std::fabs(t.wc[g][i][j]);
+      }
+    }
+    for (int k = 0; k < 2; ++k)
+      if (!(c[k] < 7.99) || !(h[k] < 3.99)) return false;
+  }
+  return true;
+}
+
 int build_tables(int N, Tabs* t, bool parent) {
   if (N < 1 || N > kMaxN) return 1;
   std::memset(t, 0, sizeof(*t));
@@ -315,10 +333,8 @@ int build_tables(int N, Tabs* t, bool parent) {
       const ld h = fabsl(Gm[g][i]) / Gm[g][weno_ref(N, g)];
       t->wh[g][i] = (double)h;
       for (int j = 0; j < N; ++j) t->wc[g][i][j] = (double)(h * Eg[g][i][j]);
-      if (t->wh[g][i] >= 2.0) return 3;  // the ranges of the kernels' fixed-point sums
-      for (int j = 0; j < N; ++j)
-        if (std::fabs(t->wc[g][i][j]) >= 2.0) return 3;
     }
+  if (!sums_fit(*t, parent)) return 3;
   // subcell averages (Fig. 1): N equal parts of each neighbour, troubled cell whole
   {
     ld qx[kMaxQ], qw[kMaxQ];

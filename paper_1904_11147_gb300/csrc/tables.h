@@ -67,6 +67,11 @@ DGT_HD constexpr int weno_neg(int N, int g, bool parent) {
   return N == 3 && !parent && g == 1 ? 3 : (N == 3 && !parent && g == 2 ? 0 : -1);
 }
 
+// Whether wh and wc fit the kernels' fixed point (weno_diff): as 64-bit constants (|wc| < 2, wh < 2), and
+// in the sums over the stencils, of terms below |wc| 2^60 in 2^63 and below wh 2^61 in 2^63.  At a point
+// with a negative weight the two parts are summed apart.
+bool sums_fit(const Tabs& t, bool parent);
+
 // Fills t for degree N; returns 0 on success.  parent: the limiter tables of the parent
 // WENO limiter (whole cells j-N .. j+N) instead of CSWENO's subcells.
 int build_tables(int N, Tabs* t, bool parent = false);
