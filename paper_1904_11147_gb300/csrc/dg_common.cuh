@@ -95,21 +95,6 @@ struct Phys<DIM, 0> {  // Burgers, f = g = u^2 / 2
 };
 
 template <>
-struct Phys<1, 1> {  // 1D Euler (rho, m, E)
-  static constexpr int V = 3;
-  __device__ __forceinline__ static void flux(int, const double* u, double* f, double& a, double gam,
-                                              double gm1) {
-    double r = 1.0 / u[0];
-    double vel = u[1] * r;
-    double p = gm1 * (u[2] - 0.5 * u[1] * vel);
-    f[0] = u[1];
-    f[1] = fma(u[1], vel, p);
-    f[2] = (u[2] + p) * vel;
-    a = fabs(vel) + sqrt(gam * p * r);
-  }
-};
-
-template <>
 struct Phys<2, 1> {  // 2D Euler (rho, mx, my, E)
   static constexpr int V = 4;
   __device__ __forceinline__ static void flux(int dir, const double* u, double* f, double& a, double gam,

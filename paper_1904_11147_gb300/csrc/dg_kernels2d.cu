@@ -25,8 +25,8 @@ template <int N>
 struct Lay {
   static constexpr int Q = N + 1, NP = (N + 1) * (N + 2) / 2;
   static constexpr int N1 = N + 1;
-  static constexpr int SIZE_DG = 3 * Q * Q * NP + N1 + 2 * Q * N1;
-  static constexpr int SIZE_FLAG = 4 * NP + 1;
+  static constexpr int SIZE_DG = 2 * Q * Q * NP + N1 + 2 * Q * N1;
+  static constexpr int SIZE_FLAG = 2 * NP + 1;
   static constexpr int SIZE_PROJ = 3 * 8 + 8 * N1;
   static constexpr int SIZE = SIZE_DG + SIZE_FLAG + SIZE_PROJ;
 };
@@ -37,17 +37,14 @@ template <int N>
 struct Off {
   using L = Lay<N>;
   static constexpr int Q = L::Q, NP = L::NP, N1 = L::N1;
-  static constexpr int VP = base_of(N);          // [Q*Q][NP] psi_a(x_qx) psi_b(x_qy)
-  static constexpr int VDX = VP + Q * Q * NP;    // w w psi_a'(x_qx) psi_b(x_qy)
+  static constexpr int VDX = base_of(N);         // [Q*Q][NP] w w psi_a'(x_qx) psi_b(x_qy)
   static constexpr int VDY = VDX + Q * Q * NP;   // w w psi_a(x_qx) psi_b'(x_qy)
   static constexpr int P1 = VDY + Q * Q * NP;    // psi_n(1)
   static constexpr int PQ = P1 + N1;             // [Q][N1] psi_n(x_q)
   static constexpr int WPQ = PQ + Q * N1;        // [Q][N1] w_q psi_n(x_q)
   static constexpr int TE = WPQ + Q * N1;        // [NP] psi_a(1) psi_b(0)
-  static constexpr int TW = TE + NP;             // psi_a(-1) psi_b(0)
-  static constexpr int TN = TW + NP;             // psi_a(0) psi_b(1)
-  static constexpr int TS = TN + NP;             // psi_a(0) psi_b(-1)
-  static constexpr int C00 = TS + NP;            // psi_0(0)^2
+  static constexpr int TN = TE + NP;             // psi_a(0) psi_b(1)
+  static constexpr int C00 = TN + NP;            // psi_0(0)^2
   static constexpr int PX = C00 + 1;             // [8]
   static constexpr int PW = PX + 8;              // [8]
   static constexpr int PQP = PW + 8;             // [8] (count in slot 0)
@@ -71,7 +68,6 @@ void pack(const dgt::Tabs& t, double* h) {
       for (int m = 0; m < NP; ++m) {
         int a = mode_a(m), b = mode_b(m), q = qy * Q + qx;
         double ww = t.gw[qx] * t.gw[qy];
-        h[O::VP + q * NP + m] = t.psi_q[qx][a] * t.psi_q[qy][b];
         h[O::VDX + q * NP + m] = ww * t.dpsi_q[qx][a] * t.psi_q[qy][b];
         h[O::VDY + q * NP + m] = ww * t.psi_q[qx][a] * t.dpsi_q[qy][b];
       }
@@ -84,9 +80,7 @@ void pack(const dgt::Tabs& t, double* h) {
   for (int m = 0; m < NP; ++m) {
     int a = mode_a(m), b = mode_b(m);
     h[O::TE + m] = t.psi_p1[a] * t.psi_0[b];
-    h[O::TW + m] = t.psi_m1[a] * t.psi_0[b];
     h[O::TN + m] = t.psi_0[a] * t.psi_p1[b];
-    h[O::TS + m] = t.psi_0[a] * t.psi_m1[b];
   }
   h[O::C00] = t.psi_0[0] * t.psi_0[0];
   for (int q = 0; q < t.QP; ++q) {

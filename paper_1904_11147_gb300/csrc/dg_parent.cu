@@ -1,14 +1,13 @@
 // Parent WENO limiter (Qiu and Shu, ref. [qs1]; the limiter the paper compares CSWENO
-// with in Sec. 4): the reconstruction of Sec. 3, Steps 2-6, on the averages of the whole
-// cells j-N .. j+N instead of subcells of the immediate neighbours.  In 2D: dimension by
-// dimension on the (2N+1)^2 cell averages around the troubled cell (x sweep, then y sweep,
-// tensor projection), characteristic fields with the x (y) Jacobian eigenvectors at the
-// troubled cell's mean for Euler.  Outflow ghosts mirror the interior cell at the
-// reflected position (ghost -1-k <-> cell k; a mirror image keeps the mean).
+// with in Sec. 4) in 1D: the reconstruction of Sec. 3, Steps 2-6, on the averages of the whole
+// cells j-N .. j+N instead of subcells of the immediate neighbours, in characteristic
+// fields at the troubled cell's mean for Euler (the 2D one is in dg_limit2.cu).  Outflow ghosts
+// mirror the interior cell at the reflected position (ghost -1-k <-> cell k; a mirror image
+// keeps the mean).
 //
 // One thread per listed (troubled) cell, the same compacted list and compact output
 // buffer as the CSWENO kernels; the scatter kernel writes the result back (Jacobi).
-// Only cell means are read from the neighbourhood: (2N+1)^dim cells x V values.
+// Only cell means are read from the neighbourhood: 2N+1 cells x V values.
 #include "dg_shared.cuh"
 #include "tables.h"
 
@@ -22,7 +21,7 @@ struct PTab {
   double gpn[4][4], gmn[4][4], sgp[4], sgm[4], neg[4];  // split of negative weights
   double pg[4][4];      // psi_n at the reconstruction points [g][n]
   double wg[4];         // their quadrature weights
-  double psi0;          // psi_0 (cell mean = U_0 psi_0 in 1D, U_00 psi_0^2 in 2D)
+  double psi0;          // psi_0 (cell mean = U_0 psi_0)
 };
 
 __constant__ PTab c_pt[3];
@@ -99,39 +98,20 @@ __device__ __forceinline__ void weno_p(const PTab& t, const double* avg, double*
   }
 }
 
-// right (R) and left (L) eigenvectors of the Euler flux Jacobian at the mean state u:
-// 1D (V = 3), or 2D (V = 4) in direction dir
-template <int V>
-__device__ __forceinline__ void eig(const double* u, int dir, double gam, double (&R)[V][V], double (&L)[V][V]) {
+// right (R) and left (L) eigenvectors of the 1D Euler flux Jacobian at the mean state u
+__device__ __forceinline__ void eig(const double (&u)[3], double gam, double (&R)[3][3], double (&L)[3][3]) {
   const double rho = u[0], r = 1.0 / rho;
-  const double vx = u[1] * r, vy = V == 4 ? u[2] * r : 0.0, q2 = vx * vx + vy * vy;
-  const double p = (gam - 1.0) * (u[V - 1] - 0.5 * rho * q2);
+  const double vx = u[1] * r, q2 = vx * vx;
+  const double p = (gam - 1.0) * (u[2] - 0.5 * rho * q2);
   const double c = sqrt(gam * p * r), ic = 1.0 / c;
-  const double H = (u[V - 1] + p) * r;
+  const double H = (u[2] + p) * r;
   const double b1 = (gam - 1.0) * ic * ic, b2 = 0.5 * b1 * q2;
-#pragma unroll
-  for (int i = 0; i < V; ++i)
-#pragma unroll
-    for (int j = 0; j < V; ++j) { R[i][j] = 0.0; L[i][j] = 0.0; }
-  if constexpr (V == 3) {
-    R[0][0] = 1.0; R[1][0] = vx - c; R[2][0] = H - vx * c;
-    R[0][1] = 1.0; R[1][1] = vx;     R[2][1] = 0.5 * q2;
-    R[0][2] = 1.0; R[1][2] = vx + c; R[2][2] = H + vx * c;
-    L[0][0] = 0.5 * (b2 + vx * ic); L[0][1] = -0.5 * (b1 * vx + ic); L[0][2] = 0.5 * b1;
-    L[1][0] = 1.0 - b2;             L[1][1] = b1 * vx;               L[1][2] = -b1;
-    L[2][0] = 0.5 * (b2 - vx * ic); L[2][1] = 0.5 * (ic - b1 * vx);  L[2][2] = 0.5 * b1;
-  } else {
-    const double vn = dir == 0 ? vx : vy, vt = dir == 0 ? vy : vx;
-    const int in = dir == 0 ? 1 : 2, it = dir == 0 ? 2 : 1;
-    R[0][0] = 1.0; R[in][0] = vn - c; R[it][0] = vt; R[3][0] = H - vn * c;
-    R[0][1] = 1.0; R[in][1] = vn;     R[it][1] = vt; R[3][1] = 0.5 * q2;
-    R[it][2] = 1.0; R[3][2] = vt;
-    R[0][3] = 1.0; R[in][3] = vn + c; R[it][3] = vt; R[3][3] = H + vn * c;
-    L[0][0] = 0.5 * (b2 + vn * ic); L[0][in] = -0.5 * (b1 * vn + ic); L[0][it] = -0.5 * b1 * vt; L[0][3] = 0.5 * b1;
-    L[1][0] = 1.0 - b2;             L[1][in] = b1 * vn;               L[1][it] = b1 * vt;        L[1][3] = -b1;
-    L[2][0] = -vt;                  L[2][it] = 1.0;
-    L[3][0] = 0.5 * (b2 - vn * ic); L[3][in] = 0.5 * (ic - b1 * vn);  L[3][it] = -0.5 * b1 * vt; L[3][3] = 0.5 * b1;
-  }
+  R[0][0] = 1.0; R[1][0] = vx - c; R[2][0] = H - vx * c;
+  R[0][1] = 1.0; R[1][1] = vx;     R[2][1] = 0.5 * q2;
+  R[0][2] = 1.0; R[1][2] = vx + c; R[2][2] = H + vx * c;
+  L[0][0] = 0.5 * (b2 + vx * ic); L[0][1] = -0.5 * (b1 * vx + ic); L[0][2] = 0.5 * b1;
+  L[1][0] = 1.0 - b2;             L[1][1] = b1 * vx;               L[1][2] = -b1;
+  L[2][0] = 0.5 * (b2 - vx * ic); L[2][1] = 0.5 * (ic - b1 * vx);  L[2][2] = 0.5 * b1;
 }
 
 // one sweep: averages a[v][k] (k over the 2N+1 stencil cells) -> point values o[v][g],
@@ -192,7 +172,7 @@ __global__ void __launch_bounds__(128)
       double mean[V];
 #pragma unroll
       for (int v = 0; v < V; ++v) mean[v] = a[v][N];
-      eig<V>(mean, 0, gam, R, L);
+      eig(mean, gam, R, L);
     }
     double val[V][NG];
     sweep<PDE, V, N>(t, a, R, L, val);

@@ -171,7 +171,6 @@ int build_tables(int N, Tabs* t, bool parent) {
   }
   for (int n = 0; n <= N; ++n) {
     t->psi_p1[n] = (double)psi(n, 1.0L);
-    t->kp1[n] = (double)(sqrtl(2.0L) * psi(n, 1.0L));
     t->kp1_fix[n] = llrintl(ldexpl(sqrtl(2.0L) * psi(n, 1.0L), 61));
     t->psi_m1[n] = (double)psi(n, -1.0L);
     t->psi_0[n] = (double)psi(n, 0.0L);
