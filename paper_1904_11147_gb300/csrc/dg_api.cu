@@ -59,7 +59,7 @@ void launch_label(int dim, int pde, int N, const LaunchArgs& a, double c0, const
                   const Counters* cnt, const double* lim, float* label, int nblocks);
 long long mlp_wgrad_chunks(long long B);
 void launch_mlp_grad(cudaStream_t st, const float* X, const unsigned char* y, long long B, int F, const float* params,
-                     float pw, float* part, float* loss, float* grad);
+                     float pw, float* part, float* grad);
 void launch_mlp_forward(cudaStream_t st, const float* X, long long B, int F, const float* params, float* z);
 void launch_mlp_adam(cudaStream_t st, float* params, const float* grad, float* m1, float* m2, int P, float lr, int t);
 void launch_mlp_export(cudaStream_t st, const float* params, int F, int FP, void* W1b, float* b1, void* W2b, float* b2,
@@ -1332,10 +1332,10 @@ extern "C" dg_status dg_limiter_tables(int N, double* rp, double* rw, double* C,
 struct dg_mlp {
   int F = 0, FP = 0, P = 0, t = 0;
   cudaStream_t st = nullptr;
-  float *params = nullptr, *grad = nullptr, *m1 = nullptr, *m2 = nullptr, *loss = nullptr;
+  float *params = nullptr, *grad = nullptr, *m1 = nullptr, *m2 = nullptr;  // grad [P + 1]: the loss behind it
   void* infer = nullptr;  // BF16 W1 [32][FP], BF16 W2 [32][32], FP32 b1, b2, w3, b3
   long long cap = 0;
-  float* part = nullptr;  // per-chunk weight gradients [chunks][P]
+  float* part = nullptr;  // per-chunk weight gradients and loss [chunks][P + 1]
 };
 
 static const int kHidden = 32;
@@ -1373,7 +1373,7 @@ extern "C" size_t dg_mlp_param_count(const dg_mlp* n) { return n ? (size_t)n->P 
 
 extern "C" dg_status dg_mlp_destroy(dg_mlp* n) {
   if (!n) return DG_OK;
-  cudaFree(n->params); cudaFree(n->grad); cudaFree(n->m1); cudaFree(n->m2); cudaFree(n->loss); cudaFree(n->infer);
+  cudaFree(n->params); cudaFree(n->grad); cudaFree(n->m1); cudaFree(n->m2); cudaFree(n->infer);
   cudaFree(n->part);
   delete n;
   return DG_OK;
@@ -1390,9 +1390,9 @@ extern "C" dg_status dg_mlp_create(int n_features, uint64_t seed, void* stream, 
   n->P = kHidden * n_features + kHidden + kHidden * kHidden + kHidden + kHidden + 1;
   n->st = (cudaStream_t)stream;
   const size_t pb = sizeof(float) * n->P;
-  if (cudaMalloc(&n->params, pb) != cudaSuccess || cudaMalloc(&n->grad, pb) != cudaSuccess ||
+  if (cudaMalloc(&n->params, pb) != cudaSuccess || cudaMalloc(&n->grad, pb + sizeof(float)) != cudaSuccess ||
       cudaMalloc(&n->m1, pb) != cudaSuccess || cudaMalloc(&n->m2, pb) != cudaSuccess ||
-      cudaMalloc(&n->loss, sizeof(float)) != cudaSuccess || cudaMalloc(&n->infer, infer_bytes(n->FP)) != cudaSuccess) {
+      cudaMalloc(&n->infer, infer_bytes(n->FP)) != cudaSuccess) {
     cudaGetLastError();
     dg_mlp_destroy(n);
     return fail(DG_ENOMEM, "device allocation for the network");
@@ -1451,15 +1451,14 @@ static dg_status mlp_backward(dg_mlp* n, const float* X, const uint8_t* y, int64
   if (B > n->cap) {
     cudaFree(n->part);
     n->part = nullptr;
-    if (cudaMalloc(&n->part, sizeof(float) * (size_t)n->P * (size_t)mlp_wgrad_chunks(B)) != cudaSuccess) {
+    if (cudaMalloc(&n->part, sizeof(float) * (size_t)(n->P + 1) * (size_t)mlp_wgrad_chunks(B)) != cudaSuccess) {
       cudaGetLastError();
       n->cap = 0;
       return fail(DG_ENOMEM, "training scratch for %lld samples", (long long)B);
     }
     n->cap = B;
   }
-  CK(cudaMemsetAsync(n->loss, 0, sizeof(float), n->st));
-  launch_mlp_grad(n->st, X, y, B, n->F, n->params, pw, n->part, n->loss, n->grad);
+  launch_mlp_grad(n->st, X, y, B, n->F, n->params, pw, n->part, n->grad);
   CK(cudaGetLastError());
   return DG_OK;
 }
@@ -1470,7 +1469,7 @@ extern "C" dg_status dg_mlp_grad(dg_mlp* n, const float* X, const uint8_t* y, in
   dg_status s = mlp_backward(n, X, y, B, pos_weight);
   if (s != DG_OK) return s;
   if (grad_out) CK(cudaMemcpyAsync(grad_out, n->grad, sizeof(float) * n->P, cudaMemcpyDeviceToHost, n->st));
-  if (loss_out) CK(cudaMemcpyAsync(loss_out, n->loss, sizeof(float), cudaMemcpyDeviceToHost, n->st));
+  if (loss_out) CK(cudaMemcpyAsync(loss_out, n->grad + n->P, sizeof(float), cudaMemcpyDeviceToHost, n->st));
   CK(cudaStreamSynchronize(n->st));
   return DG_OK;
 }
@@ -1485,7 +1484,7 @@ extern "C" dg_status dg_mlp_train_step(dg_mlp* n, const float* X, const uint8_t*
   mlp_export(n);
   CK(cudaGetLastError());
   if (loss_out) {
-    CK(cudaMemcpyAsync(loss_out, n->loss, sizeof(float), cudaMemcpyDeviceToHost, n->st));
+    CK(cudaMemcpyAsync(loss_out, n->grad + n->P, sizeof(float), cudaMemcpyDeviceToHost, n->st));
     CK(cudaStreamSynchronize(n->st));
   }
   return DG_OK;

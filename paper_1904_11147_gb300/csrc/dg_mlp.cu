@@ -569,8 +569,8 @@ __global__ void k_label(const double* __restrict__ U, const Inst* __restrict__ i
 
 // ----------------------------------------------------------------------------- training
 // Loss and weight gradients of a chunk of samples: forward pass, backpropagated deltas and
-// part[chunk][p] = sum_b delta[b][o] input[b][i] over the chunk; k_mlp_wsum adds the chunks in
-// a fixed order, so that training is reproducible bit for bit.  (Sums run over features,
+// part[chunk][p] = sum_b delta[b][o] input[b][i] over the chunk, behind them (p = P) its part of the
+// loss; k_mlp_wsum adds the chunks in a fixed order, so that training is reproducible bit for bit.  (Sums run over features,
 // hidden units and samples in ascending order.)
 //
 // One block per chunk of 64 samples: lane = sample, and a warp holds 8 of the 32 hidden units
@@ -583,13 +583,13 @@ constexpr int kChunk = 64, kSlice = 32, kPad = 36;
 
 __global__ void __launch_bounds__(256)
     k_mlp_grad(const float* __restrict__ X, const unsigned char* __restrict__ y, long long B, int F,
-               const float* __restrict__ params, float pw, float* __restrict__ part, float* __restrict__ loss_acc) {
+               const float* __restrict__ params, float pw, float* __restrict__ part) {
   __shared__ __align__(16) float sX[kChunk * (kSlice + 1)];
   __shared__ __align__(16) float sWD[kChunk * kPad];  // slice of W1, transposed; then the deltas of layer 1
   __shared__ __align__(16) float sH1[kChunk * (kHid + 1)];
   __shared__ __align__(16) float sA[kChunk * kPad];   // layer 2's output, then its deltas
   __shared__ __align__(16) float sW2[kHid * kPad], sW2T[kHid * kPad];
-  __shared__ float sb1[kHid], sb2[kHid], sw3[kHid], sdz[kChunk];
+  __shared__ float sb1[kHid], sb2[kHid], sw3[kHid], sdz[kChunk], sloss[2];
   const float* const gW2 = params + kHid * F + kHid;
   const float* const gb2 = gW2 + kHid * kHid;
   const float* const gw3 = gb2 + kHid;
@@ -597,7 +597,7 @@ __global__ void __launch_bounds__(256)
   const long long b0 = (long long)blockIdx.x * kChunk;
   const int nb = (int)min((long long)kChunk, B - b0);
   const int P = kHid * F + kHid + kHid * kHid + kHid + kHid + 1;
-  float* const out = part + (long long)blockIdx.x * P;
+  float* const out = part + (long long)blockIdx.x * (P + 1);
   for (int k = tid; k < kHid * kHid; k += 256) {
     const float v = gW2[k];
     sW2[(k / kHid) * kPad + k % kHid] = v;
@@ -663,13 +663,14 @@ __global__ void __launch_bounds__(256)
   const float dz = (pw * yy * (sig - 1.f) + (1.f - yy) * sig) / (float)B;
   if (o0 == 0) {
     sdz[s] = dz;
-    // loss: warp sum then one atomic per warp
+    // loss: a sum per warp
     float lossv = s < nb ? pw * yy * spn + (1.f - yy) * spz : 0.f;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) lossv += __shfl_xor_sync(0xffffffffu, lossv, o);
-    if (lane == 0 && s < nb) atomicAdd(loss_acc, lossv / (float)B);
+    if (lane == 0) sloss[w] = lossv;
   }
   __syncthreads();
+  if (tid == kHid + 1) out[P] = (sloss[0] + sloss[1]) / (float)B;
   if (tid <= kHid) {  // w3, b3
     float t = 0.f;
     for (int j = 0; j < nb; ++j) t = tid < kHid ? fmaf(sdz[j], sA[j * kPad + (tid < kHid ? tid : 0)], t) : t + sdz[j];
@@ -774,6 +775,7 @@ __global__ void k_mlp_forward(const float* __restrict__ X, long long B, int F, c
 // The chunks' gradients added in order, with the rounding errors of the sum carried along: 8192
 // samples make 128 chunks, and a plain FP32 sum of their gradients was off by 4e-7 (against
 // 64 bits; 6.5e-8 with the errors carried).  It costs no measurable time: the loads bound it.
+// P: columns of part, the loss included.
 __global__ void k_mlp_wsum(const float* __restrict__ part, int nchunks, int P, float* __restrict__ grad) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= P) return;
@@ -958,11 +960,11 @@ void launch_mlp_forward(cudaStream_t st, const float* X, long long B, int F, con
 long long mlp_wgrad_chunks(long long B) { return (B + kChunk - 1) / kChunk; }
 
 void launch_mlp_grad(cudaStream_t st, const float* X, const unsigned char* y, long long B, int F, const float* params,
-                     float pw, float* part, float* loss, float* grad) {
+                     float pw, float* part, float* grad) {
   const long long nc = mlp_wgrad_chunks(B);
   const int P = kHid * F + kHid + kHid * kHid + kHid + kHid + 1;
-  k_mlp_grad<<<(unsigned)nc, 256, 0, st>>>(X, y, B, F, params, pw, part, loss);
-  k_mlp_wsum<<<(P + 127) / 128, 128, 0, st>>>(part, (int)nc, P, grad);
+  k_mlp_grad<<<(unsigned)nc, 256, 0, st>>>(X, y, B, F, params, pw, part);
+  k_mlp_wsum<<<(P + 128) / 128, 128, 0, st>>>(part, (int)nc, P + 1, grad);
 }
 
 void launch_mlp_adam(cudaStream_t st, float* params, const float* grad, float* m1, float* m2, int P, float lr,
