@@ -128,8 +128,10 @@ dg_status dg_set_dt(dg_mesh* m, const double* dt);
  *   stage 3: u^{n+1} = 1/3 u^n + 2/3 (u2 + dt L(u2))
  * L is evaluated on the current state (the previous stage, limited or not).  dt > 0 applies
  * to every instance; dt <= 0 uses the per-instance values of dg_set_dt.  No limiting.
- * FP64 arithmetic; in 2D Euler the reciprocal of the density and the sound speed's square
- * root are the hardware's approximations refined to within 1-2 ulp of the IEEE results.
+ * FP64 arithmetic; for Euler the reciprocal of the density and the sound speed's square
+ * root are the hardware's approximations refined to within 1-2 ulp of the IEEE results.  The
+ * split 2D stage forms the traces (P2: also the volume's point values) as 64-bit fixed-point sums
+ * over the variable's largest mode, rounded once (at most 4.3e-17 of that mode off before it).
  * Errors: DG_EINVAL (stage not 1..3), DG_ESTATE (stage s without stage s-1 before it). */
 dg_status dg_rk_stage(dg_mesh* m, int stage, double dt);
 
@@ -155,8 +157,10 @@ dg_status dg_flag_cells(dg_mesh* m, int indicator, double tvb_M, int64_t* n_flag
  * dg_flag_cells: keeps each troubled cell's average U_0 and rebuilds modes 1..N from WENO
  * point values reconstructed on the subcells of its immediate neighbours (characteristic
  * fields for Euler; dimension by dimension in 2D).  Jacobi update: every troubled cell
- * reads the unlimited neighbours.  In 2D the reciprocals in the nonlinear weights
- * (Eq. (14)) are the hardware's approximations refined to within 1-2 ulp.  After the
+ * reads the unlimited neighbours.  The nonlinear weights' products (Eq. (14)) carry 64-bit
+ * significands and the sums over the stencils are formed in 64-bit fixed point over their
+ * largest term; the quotient is rounded once in 2D, and in 1D a product with a reciprocal
+ * refined to within 1-2 ulp.  After the
  * learned indicator's flags (Euler) the positivity fallback of dg_set_indicator_mlp applies
  * as in dg_step.  Errors: DG_ESTATE if no flags exist for this state. */
 dg_status dg_cswenolimit(dg_mesh* m);

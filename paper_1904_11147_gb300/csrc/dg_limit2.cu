@@ -13,13 +13,13 @@
 // 2N+1 averages.  Structural zeros of the subcell averages are used (a half of a cell has
 // no part of an even mode, a whole cell only that of psi_0), and the arithmetic has the
 // three-register form of dg_weno.cuh, whose reconstruction leaves only the smoothness
-// indicators and the final quotients to the FP64 pipe.
+// indicators to the FP64 pipe (the quotients are formed in integers, too).
 //
 // Per troubled cell of a 512^2 Euler mesh (half its cells troubled): P2 4.0 ns, P3 8.9 ns.  With FP64
 // quotients and dense subcell sums: 5.1 and 11; with the line reconstruction inlined in
 // both sweeps: 5.6 and 14; with it wholly in FP64 besides: 7.4 and 16; on averages instead of
 // differences, with a reciprocal per stencil: 13 and 28.  The FP64 pipe is busy 82 % (P2) and
-// 68 % (P3) of the time; the rest is the latency of the integer chains at 12 to 15 warps per SM.
+// 69 % (P3) of the time; the rest is the latency of the integer chains at 12 to 15 warps per SM.
 #include "dg_shared.cuh"
 #include "dg_weno.cuh"
 

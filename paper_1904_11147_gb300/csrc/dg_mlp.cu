@@ -570,8 +570,8 @@ __global__ void k_label(const double* __restrict__ U, const Inst* __restrict__ i
 // ----------------------------------------------------------------------------- training
 // Loss and weight gradients of a chunk of samples: forward pass, backpropagated deltas and
 // part[chunk][p] = sum_b delta[b][o] input[b][i] over the chunk, behind them (p = P) its part of the
-// loss; k_mlp_wsum adds the chunks in a fixed order, so that training is reproducible bit for bit.  (Sums run over features,
-// hidden units and samples in ascending order.)
+// loss; k_mlp_wsum adds the chunks in a fixed order, so that training is reproducible bit for bit.
+// (Sums run over features, hidden units and samples in ascending order.)
 //
 // One block per chunk of 64 samples: lane = sample, and a warp holds 8 of the 32 hidden units
 // of its 32 samples.  Features pass through shared memory in slices of 32, loaded coalesced
@@ -773,8 +773,9 @@ __global__ void k_mlp_forward(const float* __restrict__ X, long long B, int F, c
 }
 
 // The chunks' gradients added in order, with the rounding errors of the sum carried along: 8192
-// samples make 128 chunks, and a plain FP32 sum of their gradients was off by 4e-7 (against
-// 64 bits; 6.5e-8 with the errors carried).  It costs no measurable time: the loads bound it.
+// samples make 128 chunks, and a plain FP32 sum of their gradients is off by 1.3e-7 (of the largest
+// component, against 64 bits; 6.5e-8, most of it from within the chunks, with the errors carried).
+// It costs no measurable time: the loads bound it.
 // P: columns of part, the loss included.
 __global__ void k_mlp_wsum(const float* __restrict__ part, int nchunks, int P, float* __restrict__ grad) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;

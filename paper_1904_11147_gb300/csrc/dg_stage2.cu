@@ -22,7 +22,7 @@
 // 32-wide face tiles): 1024^2 P2 face pass 0.70 ms (0.87, 1.09), cell pass 0.81 ms (0.88,
 // 1.19); P3 batch of 1.10 M cells 1.04 ms (1.46, 1.84) and 1.98 ms (1.98, 3.18); 1537 x 1021 P1
 // 0.68 ms (0.80, 1.02) and 0.44 ms (0.44, 0.66).  With the traces in one function the face pass is
-// 8 % (P2) and 16 % (P3) faster still: 512^2 0.18 and 0.24 ms, the FP64 pipe 85 % busy.
+// 8 % (P2) and 16 % (P3) faster still: 512^2 0.18 and 0.25 ms, the FP64 pipe 84 % busy.
 #include <cmath>
 #include <cstring>
 
@@ -283,7 +283,10 @@ __global__ void __launch_bounds__(kFaceChunk) k_face2(const double* __restrict__
 // Two blocks per SM (at most 128 registers) except for Euler P3; Euler P2 and P3 keep the cell's
 // modes in shared memory (one slot per thread and mode).  Point values in fixed point pay for
 // P2 (Euler 878 -> 809 us at 1024^2, Burgers 211 -> 198 us); P1 has too little to move (439 -> 470 us)
-// and P3 no registers for it (1.98 -> 2.74 ms): those stay in FP64.
+// and P3 no registers for it (1.98 -> 2.74 ms): those stay in FP64.  Euler P2 pays for it with
+// register spills (588 B stored and 836 B loaded per thread; 104 and 116 B with FP64 values, plain
+// sums and no modes in shared memory) and a second read of the modes for the combination; one
+// block per SM, with room for both, is no faster (13.5 against 13.3 ms per 1024^2 step).
 __host__ __device__ constexpr bool fixed_values(int N) { return N == 2; }
 __host__ __device__ constexpr bool smem_modes(int pde, int N) { return pde == 1 && N >= 2; }
 

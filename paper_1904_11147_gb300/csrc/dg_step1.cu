@@ -474,7 +474,8 @@ __global__ void __launch_bounds__(128)
 // most of the block's warps idle.
 // Measured per step, with five kernels per stage in parentheses: 160 Burgers P2 cells 21 us
 // (80), 64 x 800 Euler P3 cells 180 us (468).  Three blocks per SM (448 tiles of the latter on
-// 152 SMs) bound the registers to 168; tiles of 84 cells would need a second wave.
+// 152 SMs) bound the registers to 168; tiles of 84 cells would need a second wave.  (Other batches were
+// not measured for the tile's size.)  P3 spills some 350 B per thread at that bound.
 constexpr int kStepThreads = 128, kHalo = 6, kStepTile = kStepThreads - 2 * kHalo;
 
 template <int PDE, int N>
